@@ -115,3 +115,14 @@ def test_guided_schedules_zero_weights(torch, B):
                              1).cpu().numpy()
     assert np.array_equal(got, O.guided_schedules(d, 5, 0.0, 1, rnd))
     assert np.all(got[:, 1, 3] == 1) and np.all(got[:, 2, 7] == 1)
+
+
+@pytest.mark.parametrize("units,steps,K", [(1, 1, 1), (3, 10, 30), (1, 33, 7), (5, 51, 255), (24, 100, 240), (32, 128, 500)])
+def test_guided_schedules_run_edges(torch, B, units, steps, K):
+    # fewer cells than lanes, runs that do not divide the cells, every cell drawn, the largest lattice
+    rng = np.random.default_rng(units * steps)
+    d = (rng.random((units, steps)) + 0.01).astype(np.float32)
+    rnd = synth.guided_randoms(3, K, 9)
+    got = B.guided_schedules(torch.from_numpy(d).cuda(), K, torch.from_numpy(rnd.view(np.int64)).cuda(), 0.05,
+                             2).cpu().numpy()
+    assert np.array_equal(got, O.guided_schedules(d, K, 0.05, 2, rnd))
