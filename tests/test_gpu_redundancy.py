@@ -126,3 +126,26 @@ def test_guided_schedules_run_edges(torch, B, units, steps, K):
     got = B.guided_schedules(torch.from_numpy(d).cuda(), K, torch.from_numpy(rnd.view(np.int64)).cuda(), 0.05,
                              2).cpu().numpy()
     assert np.array_equal(got, O.guided_schedules(d, K, 0.05, 2, rnd))
+
+
+@pytest.mark.parametrize("n", [64, 128, 256, 512, 1024, 2048, 4096, 8192, 16384])
+def test_map_w1_row_lengths(torch, B, n):
+    # every register-sort size (several rows per block and one) and the shared-memory sort below them;
+    # a last block with idle rows
+    rng = np.random.default_rng(n)
+    T, U, N = 4, 3, 1
+    trace = rng.standard_normal((T, U, N, n)).astype(np.float32)
+    trace[1, 0, 0, : n // 2] = 0.0                                  # ties
+    trace[2, 1, 0] = -np.abs(trace[2, 1, 0])
+    got = B.redundancy_map(torch.from_numpy(trace).cuda(), "w1").cpu().numpy()
+    _close(got, O.redundancy_map(trace.transpose(2, 1, 0, 3).astype(np.float64), "w1"))
+
+
+def test_map_w1_keeps_nan_and_inf(torch, B):
+    # a sort that lost a NaN would give its row, and every row's mean, finite values
+    rng = np.random.default_rng(3)
+    trace = rng.standard_normal((4, 3, 1, 256)).astype(np.float32)
+    trace[2, 0, 0, 17] = np.nan
+    trace[1, 1, 0, 200] = np.inf
+    got = B.redundancy_map(torch.from_numpy(trace).cuda(), "w1").cpu().numpy()
+    assert np.all(np.isnan(got[0])) and np.all(np.isinf(got[1])) and np.all(np.isfinite(got[2]))
