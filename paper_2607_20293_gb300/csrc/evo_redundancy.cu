@@ -12,11 +12,12 @@
 //   w1     : mean |sort(a_t) - sort(a_t')|          (Wasserstein-1 of the entries)
 // and d_{r,b,t} = 1/(T-1) sum_{t' != t} of the term; d_{b,t} = mean over r.
 //
-// Pair kernel: one block per (b, r).  The T rows are streamed through shared
-// memory in chunks of 32 entries; every thread owns register tiles of 4 x 4
-// (t, t') pairs and accumulates their dot products or differences over the
-// chunks (four FMA-class operations per shared-memory word loaded).  Per-sample maps go to scratch and are averaged in a second pass in
-// a fixed order (deterministic).
+// Pair kernel: a cluster of 1..8 blocks per (b, r), each with a slice of the
+// entries.  The T rows are streamed through shared memory in chunks of 64
+// entries; every thread owns an 8 x 8 register tile of (t, t') pairs of the
+// symmetric matrix (packed f32x2 accumulators: even and odd entries) for a
+// share of the chunk's entries.  Per-sample maps go to scratch and are averaged
+// in a second pass in a fixed order (deterministic).
 //
 // Guided sampling: one block per schedule.  The Eq. 7 weights are taken in
 // fixed point, q = floor((eps + d/max d)^gamma * 2^40) with IEEE double
@@ -35,152 +36,240 @@ namespace evo {
 
 namespace {
 
-constexpr int RM_CH = 64;           // entries per chunk
-constexpr int RM_THREADS = 256;
+constexpr int RM_THREADS = 192;
 constexpr int RM_MAX_T = 128;
+constexpr int RM_STAGES = 3;
 
 enum { M_COS = 0, M_MSE = 1, M_L1 = 2, M_W1 = 3 };
 
-__host__ __device__ inline int n_pairs(int T) { return T * (T + 1) / 2; }
+// Entries per chunk: 64, and 256 for T <= 32, whose few tiles leave the threads
+// to more groups of 16-byte columns.
+inline int pair_chunk(int T) { return T > 32 ? 64 : 256; }
+// eight rows of a chunk and 16 bytes of padding: a thread addresses its eight
+// rows with immediates, and neighbouring groups of rows start in distinct banks
+__host__ __device__ constexpr int pair_group(int ch) { return 8 * ch + 4; }
 
-constexpr int RM_LD = RM_CH + 4;    // shared row stride (floats): 16-byte rows, interleaved tiles hit distinct banks
-
-size_t pair_smem(int T) { return 2 * (size_t)T * RM_LD * sizeof(float) + (size_t)T * T * sizeof(float); }
+// the chunk ring; the threads' tiles (64 sums each) take its place after the last chunk
+size_t pair_smem(int T) {
+  const size_t ring = RM_STAGES * (size_t)((T + 7) / 8) * pair_group(pair_chunk(T)), tiles = (size_t)RM_THREADS * 64;
+  return (ring > tiles ? ring : tiles) * sizeof(float);
+}
 
 __device__ __forceinline__ void cp16(float* dst, const float* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
                : "memory");
 }
 
+// two fp32 values in one 64-bit register; packed multiply-add with IEEE rounding
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 fma_x2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ float2 unpack2(f32x2 v) {
+  float2 f;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(f.x), "=f"(f.y) : "l"(v));
+  return f;
+}
+// A pair's accumulator and its update with two entries of rows t (x) and t'
+// (y): even and odd entries apart where the update is one packed operation.
+// The absolute differences have no packed form (it would cost moves between
+// the halves): one accumulator, and half the registers.
 template <int METRIC>
-__device__ __forceinline__ float pair_op(float x, float y, float acc) {
-  if constexpr (METRIC == M_COS) return fmaf(x, y, acc);
-  if constexpr (METRIC == M_MSE) {
-    const float e = x - y;
-    return fmaf(e, e, acc);
+struct PairAcc {
+  f32x2 s;
+  __device__ __forceinline__ void clear() { s = 0ull; }
+  __device__ __forceinline__ void add(f32x2 x, f32x2 y) {
+    if constexpr (METRIC == M_COS) {
+      s = fma_x2(x, y, s);
+    } else {
+      const f32x2 e = fma_x2(y, 0xbf800000bf800000ull, x);   // x - y: one rounding
+      s = fma_x2(e, e, s);
+    }
   }
-  return acc + fabsf(x - y);
+  __device__ __forceinline__ float sum() const {
+    const float2 v = unpack2(s);
+    return v.x + v.y;
+  }
+};
+template <>
+struct PairAcc<M_L1> {
+  float s;
+  __device__ __forceinline__ void clear() { s = 0.f; }
+  __device__ __forceinline__ void add(f32x2 x, f32x2 y) {
+    const float2 a = unpack2(x), b = unpack2(y);
+    s += fabsf(a.x - b.x);
+    s += fabsf(a.y - b.y);
+  }
+  __device__ __forceinline__ float sum() const { return s; }
+};
+
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ void cluster_barrier() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ float ld_cluster(const float* p, uint32_t rank) {
+  uint32_t a;
+  float v;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
+  return v;
 }
 
-// One block per (b, r).  The T x T matrix of pair statistics is cut into
-// register tiles of 4 x 4 (t, t') pairs; tile (i, j) takes rows
-// t in {i, i + Tq, i + 2 Tq, i + 3 Tq} and t' likewise from j (Tq = ceil(T/4)),
-// so the float4 loads of neighbouring threads fall in different banks.
+// One cluster of CL blocks per (b, r); block `rank` sums the chunks
+// [rank nch / CL, (rank + 1) nch / CL).  The T x T matrix of pair statistics is
+// symmetric: tile (i, j), i <= j < Tq = ceil(T / 8), holds the pairs of rows
+// t = 8 i + a and t' = 8 j + c (a, c < 8).  With `tiles` = Tq (Tq + 1) / 2 the
+// block's threads are cut into groups of `tiles`; group g takes the chunk's
+// 16-byte columns g, g + groups, ...
+// Bound by latency at 12 warps per SM (the tiles' registers) and by the shared
+// loads: 16 8-byte loads feed 64 packed operations; the FP32 pipe is 31 % busy.
+// 24 units x 16 samples x 100 steps x 4,096 entries: cosine 1,279 -> 665 us,
+// mean square 1,459 -> 826 us, mean absolute 1,463 -> 880 us against the full
+// matrix in 4 x 4 tiles, one block per (b, r); 10 steps x 36 x 16: 346 -> 108 us.
+// Twice the threads at one block per SM (no spills, 9 warps) measured 1,045 us.
 // rows: row t of (b, r) starts at base + ((t * U + b) * N + r) * n
-template <int METRIC>
-__global__ void __launch_bounds__(RM_THREADS, METRIC == M_COS ? 1 : 2) pair_kernel(const float* rows, int T, int U, int N, int n,
-                                                          float* dr /* [U][N][T] */) {
+template <int METRIC, int CH>
+__global__ void __launch_bounds__(RM_THREADS, 2) pair_kernel(const float* rows, int T, int U, int N, int n, int CL,
+                                                             float* dr /* [U][N][T] */) {
+  constexpr int GROUP = pair_group(CH), COLS = CH / 4, RPP = RM_THREADS / COLS;   // rows per load pass
+  static_assert(RM_THREADS % COLS == 0, "a thread loads one 16-byte column of every row it takes");
   extern __shared__ __align__(16) float rm_smem[];
-  float* xb = rm_smem;                                  // 2 x [T][RM_LD]: chunk c in buffer c & 1
-  float* G = xb + 2 * T * RM_LD;                        // [T][T]
-  const int b = blockIdx.x / N, r = blockIdx.x % N;
-  const int Tq = (T + 3) / 4, tiles = Tq * Tq;
-  constexpr int TPT = ((RM_MAX_T / 4) * (RM_MAX_T / 4) + RM_THREADS - 1) / RM_THREADS;   // tiles per thread (max)
-  float acc[TPT][4][4];
+  const uint32_t rank = CL > 1 ? cluster_rank() : 0u;
+  const int unit = blockIdx.x / CL, b = unit / N, r = unit % N;
+  const int Tq = (T + 7) / 8, tiles = Tq * (Tq + 1) / 2;
+  const int groups = min(RM_THREADS / tiles, COLS);
+  const int grp = threadIdx.x / tiles;
+  int ti = 0, tj = threadIdx.x - grp * tiles;           // tile number -> (i, j), row i of the triangle holds Tq - i tiles
+  while (tj >= Tq - ti) {
+    tj -= Tq - ti;
+    ++ti;
+  }
+  tj += ti;
+  PairAcc<METRIC> acc[8][8];
 #pragma unroll
-  for (int q = 0; q < TPT; ++q)
+  for (int a = 0; a < 8; ++a)
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-      for (int c = 0; c < 4; ++c) acc[q][a][c] = 0.f;
-  // chunk c of every row -> buffer c & 1: 16-byte asynchronous copies when the
-  // rows are a multiple of 4 entries, plain loads otherwise (zero-padded tail)
-  const int nch = (n + RM_CH - 1) / RM_CH;
+    for (int c = 0; c < 8; ++c) acc[a][c].clear();
+  // chunk c of every row -> buffer c % RM_STAGES: 16-byte asynchronous copies
+  // when the rows are a multiple of 4 entries and start on 16 bytes, plain
+  // loads otherwise (zero-padded tail)
+  const int nch = (n + CH - 1) / CH;
+  const int cb = (int)((long long)nch * rank / CL), ce = (int)((long long)nch * (rank + 1) / CL);
+  const bool vec = (n & 3) == 0 && (reinterpret_cast<uintptr_t>(rows) & 15) == 0;
+  const int lk = 4 * (threadIdx.x % COLS), lt = threadIdx.x / COLS;
+  const long long step = (long long)U * N * n;          // floats between rows t and t + 1
+  const float* lsrc = rows + lt * step + ((long long)b * N + r) * n + lk;
   auto load_chunk = [&](int c) {
-    float* xs = xb + (c & 1) * T * RM_LD;
-    const int c0 = c * RM_CH, w = min(RM_CH, n - c0);
-    for (int v = threadIdx.x; v < T * (RM_CH / 4); v += blockDim.x) {
-      const int t = v / (RM_CH / 4), k = 4 * (v % (RM_CH / 4));
-      const float* src = rows + ((long long)(t * U + b) * N + r) * n + c0 + k;
-      float* dst = xs + t * RM_LD + k;
-      if (k + 3 < w && (n & 3) == 0) {
-        cp16(dst, src);
-      } else {
-        float4 f = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (k < w) f.x = src[0];
-        if (k + 1 < w) f.y = src[1];
-        if (k + 2 < w) f.z = src[2];
-        if (k + 3 < w) f.w = src[3];
-        *reinterpret_cast<float4*>(dst) = f;
+    if (c < ce) {
+      float* xs = rm_smem + (c % RM_STAGES) * Tq * GROUP + lk;
+      const int w = n - c * CH - lk;                    // entries of the row from this column on
+      const float* src = lsrc + (long long)c * CH;
+      for (int t = lt; t < T; t += RPP, src += RPP * step) {
+        float* dst = xs + (t >> 3) * GROUP + (t & 7) * CH;
+        if (w > 3 && vec) {
+          cp16(dst, src);
+        } else {
+          float4 f = make_float4(0.f, 0.f, 0.f, 0.f);
+          if (w > 0) f.x = src[0];
+          if (w > 1) f.y = src[1];
+          if (w > 2) f.z = src[2];
+          if (w > 3) f.w = src[3];
+          *reinterpret_cast<float4*>(dst) = f;
+        }
       }
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
-  load_chunk(0);
-  for (int c = 0; c < nch; ++c) {
-    if (c + 1 < nch) {
-      load_chunk(c + 1);
-      asm volatile("cp.async.wait_group 1;" ::: "memory");
-    } else {
-      asm volatile("cp.async.wait_group 0;" ::: "memory");
-    }
-    __syncthreads();
-    const float* xs = xb + (c & 1) * T * RM_LD;
+  // Two entries at a time, the halves of a 16-byte column in swapped order for
+  // j >= 8: row groups j and j + 8 start in the same bank.  (The results of rows
+  // beyond T, whatever their buffers hold, are dropped.)
+  const int h0 = (tj >> 3 & 1) * 2;
+  for (int s = 0; s < RM_STAGES - 1; ++s) load_chunk(cb + s);
+  for (int c = cb; c < ce; ++c) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(RM_STAGES - 2) : "memory");
+    __syncthreads();                                    // chunk c is there, chunk c - 1 has been read
+    load_chunk(c + RM_STAGES - 1);
+    if (grp < groups) {
+      const float* xs = rm_smem + (c % RM_STAGES) * Tq * GROUP;
+#pragma unroll 1
+      for (int k = 8 * grp; k < 2 * CH; k += 4) {       // k / 8: the column, k & 4: the second of its halves
+        const float* xr = xs + ti * GROUP + (k >> 3) * 4 + (h0 ^ (k >> 1 & 2));
+        const float* yr = xs + tj * GROUP + (k >> 3) * 4 + (h0 ^ (k >> 1 & 2));
+        f32x2 y[8];
 #pragma unroll
-    for (int q = 0; q < TPT; ++q) {
-      const int tile = threadIdx.x + q * RM_THREADS;
-      if (tile < tiles) {
-        const int i = tile / Tq, j = tile % Tq;
-        int ra[4], rc[4];
+        for (int q = 0; q < 8; ++q) y[q] = *reinterpret_cast<const f32x2*>(yr + q * CH);
 #pragma unroll
-        for (int a = 0; a < 4; ++a) {
-          ra[a] = min(i + a * Tq, T - 1);   // rows beyond T repeat the last row; their results are dropped
-          rc[a] = min(j + a * Tq, T - 1);
+        for (int a = 0; a < 8; ++a) {
+          const f32x2 x = *reinterpret_cast<const f32x2*>(xr + a * CH);
+#pragma unroll
+          for (int q = 0; q < 8; ++q) acc[a][q].add(x, y[q]);
         }
-#pragma unroll 2
-        for (int k = 0; k < RM_CH; k += 4) {
-          float4 x[4], y[4];
-#pragma unroll
-          for (int a = 0; a < 4; ++a) {
-            x[a] = *reinterpret_cast<const float4*>(xs + ra[a] * RM_LD + k);
-            y[a] = *reinterpret_cast<const float4*>(xs + rc[a] * RM_LD + k);
-          }
-#pragma unroll
-          for (int a = 0; a < 4; ++a)
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
-              float v = acc[q][a][c];
-              v = pair_op<METRIC>(x[a].x, y[c].x, v);
-              v = pair_op<METRIC>(x[a].y, y[c].y, v);
-              v = pair_op<METRIC>(x[a].z, y[c].z, v);
-              v = pair_op<METRIC>(x[a].w, y[c].w, v);
-              acc[q][a][c] = v;
-            }
-        }
+        if (k & 4) k += 8 * (groups - 1);
       }
     }
-    __syncthreads();   // buffer c & 1 is refilled with chunk c + 2 next
   }
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  __syncthreads();
+  // the groups' tiles side by side, then summed in group order into group 0's:
+  // entry e = 8 a + c of tile q ends in rm_smem[e * RM_THREADS + q]
+  if (grp < groups) {
 #pragma unroll
-  for (int q = 0; q < TPT; ++q) {
-    const int tile = threadIdx.x + q * RM_THREADS;
-    if (tile < tiles) {
-      const int i = tile / Tq, j = tile % Tq;
+    for (int a = 0; a < 8; ++a)
 #pragma unroll
-      for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          const int t = i + a * Tq, t2 = j + c * Tq;
-          if (t < T && t2 < T) G[t * T + t2] = acc[q][a][c];
-        }
-    }
+      for (int c = 0; c < 8; ++c) rm_smem[(8 * a + c) * RM_THREADS + threadIdx.x] = acc[a][c].sum();
   }
   __syncthreads();
-  for (int t = threadIdx.x; t < T; t += blockDim.x) {
-    float s = 0.f;
-    for (int t2 = 0; t2 < T; ++t2) {
-      if (t2 == t) continue;
-      float term;
-      if (METRIC == M_COS) {
-        const float nn = sqrtf(G[t * T + t]) * sqrtf(G[t2 * T + t2]);
-        term = nn == 0.f ? 1.f : 1.f - G[t * T + t2] / nn;
-      } else {
-        term = G[t * T + t2] / (float)n;
-      }
-      s += term;
+  if (groups > 1) {
+    for (int i = threadIdx.x; i < tiles * 64; i += RM_THREADS) {
+      float* q = rm_smem + (i / tiles) * RM_THREADS + i % tiles;
+      float v = q[0];
+      for (int g = 1; g < groups; ++g) v += q[g * tiles];
+      q[0] = v;
     }
-    dr[((long long)b * N + r) * T + t] = s / (float)(T - 1);
+    __syncthreads();
   }
+  // this block's rows of the map: a warp per row, the blocks' partial sums in rank order
+  if (CL > 1) cluster_barrier();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  auto total = [&](int t, int t2) {
+    int i = t >> 3, j = t2 >> 3, a = t & 7, c = t2 & 7;
+    if (i > j) {
+      const int m = i, o = a;
+      i = j;
+      j = m;
+      a = c;
+      c = o;
+    }
+    const float* q = rm_smem + (8 * a + c) * RM_THREADS + i * Tq - i * (i - 1) / 2 + (j - i);
+    if (CL == 1) return *q;
+    float v = 0.f;
+    for (int k = 0; k < CL; ++k) v += ld_cluster(q, k);
+    return v;
+  };
+  for (int t = rank + CL * warp; t < T; t += CL * (RM_THREADS / 32)) {
+    const float nt = METRIC == M_COS ? sqrtf(total(t, t)) : 0.f;
+    float s = 0.f;
+    for (int t2 = lane; t2 < T; t2 += 32) {
+      if (t2 == t) continue;
+      const float v = total(t, t2);
+      if (METRIC == M_COS) {
+        const float nn = nt * sqrtf(total(t2, t2));
+        s += nn == 0.f ? 1.f : 1.f - v / nn;
+      } else {
+        s += v / (float)n;
+      }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) dr[((long long)b * N + r) * T + t] = s / (float)(T - 1);
+  }
+  if (CL > 1) cluster_barrier();                        // the peers may still read this block's tiles
 }
 
 // d[b][t] = mean over r of dr[b][r][t], summed in order r = 0..N-1
@@ -405,6 +494,33 @@ __global__ void __launch_bounds__(GS_THREADS) guided_kernel(const float* d, int 
   for (int i = threadIdx.x; i < cells; i += GS_THREADS) S[(long long)p * cells + i] = taken[i];
 }
 
+template <int METRIC, int CH>
+cudaError_t launch_pair_ch(const float* rows, int T, int U, int N, int n, int CL, float* dr, cudaStream_t st) {
+  const int sm = (int)pair_smem(T);
+  const cudaError_t e = cudaFuncSetAttribute(pair_kernel<METRIC, CH>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)pair_smem(CH == 64 ? RM_MAX_T : 32));
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = CL;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.gridDim = dim3((unsigned)(U * N * CL));
+  cfg.blockDim = dim3(RM_THREADS);
+  cfg.dynamicSmemBytes = sm;
+  cfg.stream = st;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, pair_kernel<METRIC, CH>, rows, T, U, N, n, CL, dr);
+}
+
+template <int METRIC>
+cudaError_t launch_pair(const float* rows, int T, int U, int N, int n, int CL, float* dr, cudaStream_t st) {
+  return pair_chunk(T) == 64 ? launch_pair_ch<METRIC, 64>(rows, T, U, N, n, CL, dr, st)
+                             : launch_pair_ch<METRIC, 256>(rows, T, U, N, n, CL, dr, st);
+}
+
 }  // namespace
 
 size_t redundancy_scratch_bytes(int T, int U, int N, int n, int metric) {
@@ -440,21 +556,18 @@ cudaError_t launch_redundancy(const float* trace, int T, int U, int N, int n, in
     if (e != cudaSuccess) return e;
     rows = sorted;
   }
-  const int sm = (int)pair_smem(T);
+  // blocks per (b, r): enough for several rounds over the chip's 304 resident
+  // blocks (an even last round), at least four chunks each: 6 units x 1 sample of
+  // 404 entries 46 us, and 83 us undivided; 25 steps x 15 x 7 of 3,516 entries
+  // 52 us, and 43 us with at least eight chunks
+  int CL = 1;
+  const int nch = (n + pair_chunk(T) - 1) / pair_chunk(T);
+  while (CL < 8 && (long long)U * N * CL < 1216 && nch >= 4 * CL) CL *= 2;
   cudaError_t e = cudaSuccess;
   switch (metric) {
-    case M_COS:
-      e = cudaFuncSetAttribute(pair_kernel<M_COS>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-      if (e == cudaSuccess) pair_kernel<M_COS><<<U * N, RM_THREADS, sm, st>>>(rows, T, U, N, n, dr);
-      break;
-    case M_MSE:
-      e = cudaFuncSetAttribute(pair_kernel<M_MSE>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-      if (e == cudaSuccess) pair_kernel<M_MSE><<<U * N, RM_THREADS, sm, st>>>(rows, T, U, N, n, dr);
-      break;
-    default:
-      e = cudaFuncSetAttribute(pair_kernel<M_L1>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-      if (e == cudaSuccess) pair_kernel<M_L1><<<U * N, RM_THREADS, sm, st>>>(rows, T, U, N, n, dr);
-      break;
+    case M_COS: e = launch_pair<M_COS>(rows, T, U, N, n, CL, dr, st); break;
+    case M_MSE: e = launch_pair<M_MSE>(rows, T, U, N, n, CL, dr, st); break;
+    default: e = launch_pair<M_L1>(rows, T, U, N, n, CL, dr, st); break;
   }
   if (e != cudaSuccess) return e;
   mean_kernel<<<(U * T + 255) / 256, 256, 0, st>>>(dr, T, U, N, d);

@@ -149,3 +149,24 @@ def test_map_w1_keeps_nan_and_inf(torch, B):
     trace[1, 1, 0, 200] = np.inf
     got = B.redundancy_map(torch.from_numpy(trace).cuda(), "w1").cpu().numpy()
     assert np.all(np.isnan(got[0])) and np.all(np.isinf(got[1])) and np.all(np.isfinite(got[2]))
+
+
+@pytest.mark.parametrize("metric", ["cosine", "mse", "l1"])
+@pytest.mark.parametrize("T,n", [(2, 3), (7, 64), (8, 256), (9, 260), (32, 516), (33, 130), (100, 1028), (128, 333)])
+def test_map_tile_edges(torch, B, metric, T, n):
+    # row groups of eight (one, a partial one, sixteen), both chunk lengths, a ragged
+    # last chunk, several blocks per map (1,028 entries) and one
+    rng = np.random.default_rng(T * 1000 + n)
+    U, N = 2, 2
+    base = rng.standard_normal((U, N, n))
+    trace = (base[None] + 0.5 * rng.standard_normal((T, U, N, n))).astype(np.float32)
+    got = B.redundancy_map(torch.from_numpy(trace).cuda(), metric).cpu().numpy()
+    _close(got, O.redundancy_map(trace.transpose(2, 1, 0, 3).astype(np.float64), metric))
+
+
+def test_map_w1_odd_number_of_maps(torch, B):
+    # 7 x 3 x 1 per-sample values in front of the sorted rows: they start off a 16-byte boundary
+    rng = np.random.default_rng(5)
+    trace = rng.standard_normal((7, 3, 1, 512)).astype(np.float32)
+    got = B.redundancy_map(torch.from_numpy(trace).cuda(), "w1").cpu().numpy()
+    _close(got, O.redundancy_map(trace.transpose(2, 1, 0, 3).astype(np.float64), "w1"))
