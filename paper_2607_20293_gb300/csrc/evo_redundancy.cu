@@ -12,12 +12,12 @@
 //   w1     : mean |sort(a_t) - sort(a_t')|          (Wasserstein-1 of the entries)
 // and d_{r,b,t} = 1/(T-1) sum_{t' != t} of the term; d_{b,t} = mean over r.
 //
-// Pair kernel: a cluster of 1..8 blocks per (b, r), each with a slice of the
-// entries.  The T rows are streamed through shared memory in chunks of 64
-// entries; every thread owns an 8 x 8 register tile of (t, t') pairs of the
-// symmetric matrix (packed f32x2 accumulators: even and odd entries) for a
-// share of the chunk's entries.  Per-sample maps go to scratch and are averaged
-// in a second pass in a fixed order (deterministic).
+// Pair kernels: the T rows of a (b, r) are streamed through shared memory in
+// chunks; every thread owns a register tile of (t, t') pairs of the symmetric
+// matrix.  ordered_pair_kernel (a block per (b, r)) keeps every sum in index
+// order; sorted_pair_kernel (Wasserstein-1, a cluster of 1..8 blocks per (b, r))
+// cuts the entries over blocks and threads.  Per-sample maps go to scratch and
+// are averaged in a second pass in a fixed order (deterministic).
 //
 // Guided sampling: one block per schedule.  The Eq. 7 weights are taken in
 // fixed point, q = floor((eps + d/max d)^gamma * 2^40) with IEEE double
@@ -60,51 +60,6 @@ __device__ __forceinline__ void cp16(float* dst, const float* src) {
                : "memory");
 }
 
-// two fp32 values in one 64-bit register; packed multiply-add with IEEE rounding
-typedef unsigned long long f32x2;
-__device__ __forceinline__ f32x2 fma_x2(f32x2 a, f32x2 b, f32x2 c) {
-  f32x2 d;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-  return d;
-}
-__device__ __forceinline__ float2 unpack2(f32x2 v) {
-  float2 f;
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(f.x), "=f"(f.y) : "l"(v));
-  return f;
-}
-// A pair's accumulator and its update with two entries of rows t (x) and t'
-// (y): even and odd entries apart where the update is one packed operation.
-// The absolute differences have no packed form (it would cost moves between
-// the halves): one accumulator, and half the registers.
-template <int METRIC>
-struct PairAcc {
-  f32x2 s;
-  __device__ __forceinline__ void clear() { s = 0ull; }
-  __device__ __forceinline__ void add(f32x2 x, f32x2 y) {
-    if constexpr (METRIC == M_COS) {
-      s = fma_x2(x, y, s);
-    } else {
-      const f32x2 e = fma_x2(y, 0xbf800000bf800000ull, x);   // x - y: one rounding
-      s = fma_x2(e, e, s);
-    }
-  }
-  __device__ __forceinline__ float sum() const {
-    const float2 v = unpack2(s);
-    return v.x + v.y;
-  }
-};
-template <>
-struct PairAcc<M_L1> {
-  float s;
-  __device__ __forceinline__ void clear() { s = 0.f; }
-  __device__ __forceinline__ void add(f32x2 x, f32x2 y) {
-    const float2 a = unpack2(x), b = unpack2(y);
-    s += fabsf(a.x - b.x);
-    s += fabsf(a.y - b.y);
-  }
-  __device__ __forceinline__ float sum() const { return s; }
-};
-
 __device__ __forceinline__ uint32_t cluster_rank() {
   uint32_t r;
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
@@ -128,15 +83,14 @@ __device__ __forceinline__ float ld_cluster(const float* p, uint32_t rank) {
 // block's threads are cut into groups of `tiles`; group g takes the chunk's
 // 16-byte columns g, g + groups, ...
 // Bound by latency at 12 warps per SM (the tiles' registers) and by the shared
-// loads: 16 8-byte loads feed 64 packed operations; the FP32 pipe is 31 % busy.
-// 24 units x 16 samples x 100 steps x 4,096 entries: cosine 1,279 -> 665 us,
-// mean square 1,459 -> 826 us, mean absolute 1,463 -> 880 us against the full
-// matrix in 4 x 4 tiles, one block per (b, r); 10 steps x 36 x 16: 346 -> 108 us.
-// Twice the threads at one block per SM (no spills, 9 warps) measured 1,045 us.
+// loads.  Mean absolute difference, 24 units x 16 samples x 100 steps x 4,096
+// entries: 1,463 -> 880 us against the full matrix in 4 x 4 tiles, one block
+// per (b, r).  The sorted rows alone take it: the maps of the other metrics
+// keep each pair's sum in entry order (ordered_pair_kernel).
 // rows: row t of (b, r) starts at base + ((t * U + b) * N + r) * n
-template <int METRIC, int CH>
-__global__ void __launch_bounds__(RM_THREADS, 2) pair_kernel(const float* rows, int T, int U, int N, int n, int CL,
-                                                             float* dr /* [U][N][T] */) {
+template <int CH>
+__global__ void __launch_bounds__(RM_THREADS, 2) sorted_pair_kernel(const float* rows, int T, int U, int N, int n, int CL,
+                                                                    float* dr /* [U][N][T] */) {
   constexpr int GROUP = pair_group(CH), COLS = CH / 4, RPP = RM_THREADS / COLS;   // rows per load pass
   static_assert(RM_THREADS % COLS == 0, "a thread loads one 16-byte column of every row it takes");
   extern __shared__ __align__(16) float rm_smem[];
@@ -151,11 +105,11 @@ __global__ void __launch_bounds__(RM_THREADS, 2) pair_kernel(const float* rows, 
     ++ti;
   }
   tj += ti;
-  PairAcc<METRIC> acc[8][8];
+  float acc[8][8];
 #pragma unroll
   for (int a = 0; a < 8; ++a)
 #pragma unroll
-    for (int c = 0; c < 8; ++c) acc[a][c].clear();
+    for (int c = 0; c < 8; ++c) acc[a][c] = 0.f;
   // chunk c of every row -> buffer c % RM_STAGES: 16-byte asynchronous copies
   // when the rows are a multiple of 4 entries and start on 16 bytes, plain
   // loads otherwise (zero-padded tail)
@@ -201,14 +155,17 @@ __global__ void __launch_bounds__(RM_THREADS, 2) pair_kernel(const float* rows, 
       for (int k = 8 * grp; k < 2 * CH; k += 4) {       // k / 8: the column, k & 4: the second of its halves
         const float* xr = xs + ti * GROUP + (k >> 3) * 4 + (h0 ^ (k >> 1 & 2));
         const float* yr = xs + tj * GROUP + (k >> 3) * 4 + (h0 ^ (k >> 1 & 2));
-        f32x2 y[8];
+        float2 y[8];
 #pragma unroll
-        for (int q = 0; q < 8; ++q) y[q] = *reinterpret_cast<const f32x2*>(yr + q * CH);
+        for (int q = 0; q < 8; ++q) y[q] = *reinterpret_cast<const float2*>(yr + q * CH);
 #pragma unroll
         for (int a = 0; a < 8; ++a) {
-          const f32x2 x = *reinterpret_cast<const f32x2*>(xr + a * CH);
+          const float2 x = *reinterpret_cast<const float2*>(xr + a * CH);
 #pragma unroll
-          for (int q = 0; q < 8; ++q) acc[a][q].add(x, y[q]);
+          for (int q = 0; q < 8; ++q) {
+            acc[a][q] += fabsf(x.x - y[q].x);
+            acc[a][q] += fabsf(x.y - y[q].y);
+          }
         }
         if (k & 4) k += 8 * (groups - 1);
       }
@@ -222,7 +179,7 @@ __global__ void __launch_bounds__(RM_THREADS, 2) pair_kernel(const float* rows, 
 #pragma unroll
     for (int a = 0; a < 8; ++a)
 #pragma unroll
-      for (int c = 0; c < 8; ++c) rm_smem[(8 * a + c) * RM_THREADS + threadIdx.x] = acc[a][c].sum();
+      for (int c = 0; c < 8; ++c) rm_smem[(8 * a + c) * RM_THREADS + threadIdx.x] = acc[a][c];
   }
   __syncthreads();
   if (groups > 1) {
@@ -253,23 +210,177 @@ __global__ void __launch_bounds__(RM_THREADS, 2) pair_kernel(const float* rows, 
     return v;
   };
   for (int t = rank + CL * warp; t < T; t += CL * (RM_THREADS / 32)) {
-    const float nt = METRIC == M_COS ? sqrtf(total(t, t)) : 0.f;
     float s = 0.f;
-    for (int t2 = lane; t2 < T; t2 += 32) {
-      if (t2 == t) continue;
-      const float v = total(t, t2);
-      if (METRIC == M_COS) {
-        const float nn = nt * sqrtf(total(t2, t2));
-        s += nn == 0.f ? 1.f : 1.f - v / nn;
-      } else {
-        s += v / (float)n;
-      }
-    }
+    for (int t2 = lane; t2 < T; t2 += 32)
+      if (t2 != t) s += total(t, t2) / (float)n;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if (lane == 0) dr[((long long)b * N + r) * T + t] = s / (float)(T - 1);
   }
   if (CL > 1) cluster_barrier();                        // the peers may still read this block's tiles
+}
+
+// Cosine, mean square and mean absolute difference: one block per (b, r).
+// Every pair's sum runs over the entries in index order, and every row's over
+// the steps in order, so that the map is a fixed function of the trace whatever
+// the tiling: a guided draw takes a 64-bit remainder by the sum of the weights,
+// so a map that differs in its last bits draws other schedules.  The matrix is
+// symmetric: a thread owns an RA x CB tile (rows RA i .. of t, CB j .. of t',
+// on or above the diagonal) in registers.  8 x 4 for long loops: four entries
+// take 12 16-byte loads for 128 multiply-adds.  Shorter loops have too few such
+// tiles to fill their warps: 4 x 2 up to 64 steps (50 steps x 15 units x 7
+// samples of 3,516 entries, mean square: 217 us with 8 x 4, 125 us), 2 x 2 up to
+// 32 (25 steps x 15 x 7: 211 us with 8 x 4, 72 us).
+// Groups of four rows lie 16 bytes off a multiple of 128, so neighbouring j
+// start in distinct banks.
+// Bound by FP32 issue and the shared loads.  Cosine map of 24 units x 16 samples
+// x 100 steps x 4,096 entries: 1,279 us as the full matrix in 4 x 4 tiles ->
+// 665 us in 8 x 8 packed tiles with the entries cut over blocks (which changed
+// the sums) -> 580 us.
+constexpr int OP_CH = 32, OP_STAGES = 4, OP_GROUP = 4 * OP_CH + 4;
+
+__host__ __device__ constexpr int op_groups(int T) { return (T + 7) / 8 * 2; }   // groups of four rows
+// tiles of T rows: row group i pairs with the column groups j >= i RA / CB
+__host__ __device__ constexpr int op_tiles(int T, int RA, int CB) {
+  const int nr = (T + RA - 1) / RA, f = RA / CB;
+  return f * nr * (nr + 1) / 2;
+}
+constexpr int OP_SMALL_T = 32, OP_MID_T = 64;
+constexpr int op_max_threads(int RA) { return RA == 2 ? 160 : 288; }
+static_assert(op_tiles(RM_MAX_T, 8, 4) <= op_max_threads(8) && op_tiles(OP_MID_T, 4, 2) <= op_max_threads(4) &&
+                  op_tiles(OP_SMALL_T, 2, 2) <= op_max_threads(2),
+              "a tile per thread");
+size_t op_smem(int T) {
+  const size_t ring = (size_t)OP_STAGES * op_groups(T) * OP_GROUP, mat = (size_t)T * (T | 1) + T;
+  return (ring > mat ? ring : mat) * sizeof(float);
+}
+
+template <int METRIC>
+__device__ __forceinline__ float pair_op(float x, float y, float acc) {
+  if constexpr (METRIC == M_COS) return fmaf(x, y, acc);
+  if constexpr (METRIC == M_MSE) {
+    const float e = x - y;
+    return fmaf(e, e, acc);
+  }
+  return acc + fabsf(x - y);
+}
+
+template <int METRIC, int RA, int CB>
+__global__ void __launch_bounds__(op_max_threads(RA), 2) ordered_pair_kernel(const float* rows, int T, int U, int N,
+                                                                             int n, float* dr /* [U][N][T] */) {
+  extern __shared__ __align__(16) float rm_smem[];
+  const int b = blockIdx.x / N, r = blockIdx.x % N;
+  const int ng = op_groups(T);
+  constexpr int F = RA / CB;
+  const int nr = (T + RA - 1) / RA;
+  int ti = 0, tj = threadIdx.x;                         // tile number -> (i, j); row i holds F (nr - i) tiles
+  while (ti < nr && tj >= F * (nr - ti)) {
+    tj -= F * (nr - ti);
+    ++ti;
+  }
+  const bool mine = ti < nr;
+  tj += F * ti;
+  float acc[RA][CB];
+#pragma unroll
+  for (int a = 0; a < RA; ++a)
+#pragma unroll
+    for (int c = 0; c < CB; ++c) acc[a][c] = 0.f;
+  auto row = [](int t) { return (t >> 2) * OP_GROUP + (t & 3) * OP_CH; };
+  const int nch = (n + OP_CH - 1) / OP_CH;
+  const bool vec = (n & 3) == 0 && (reinterpret_cast<uintptr_t>(rows) & 15) == 0;
+  const long long step = (long long)U * N * n;          // floats between rows t and t + 1
+  const float* base = rows + ((long long)b * N + r) * n;
+  // chunk c -> buffer c % OP_STAGES; a ragged or unaligned row by plain loads, zero-padded
+  auto load_chunk = [&](int c) {
+    if (c < nch) {
+      float* xs = rm_smem + (c % OP_STAGES) * ng * OP_GROUP;
+      const int c0 = c * OP_CH;
+      for (int v = threadIdx.x; v < T * (OP_CH / 4); v += blockDim.x) {
+        const int t = v / (OP_CH / 4), k = 4 * (v % (OP_CH / 4)), w = n - c0 - k;
+        const float* src = base + t * step + c0 + k;
+        float* dst = xs + row(t) + k;
+        if (w > 3 && vec) {
+          cp16(dst, src);
+        } else {
+          float4 f = make_float4(0.f, 0.f, 0.f, 0.f);
+          if (w > 0) f.x = src[0];
+          if (w > 1) f.y = src[1];
+          if (w > 2) f.z = src[2];
+          if (w > 3) f.w = src[3];
+          *reinterpret_cast<float4*>(dst) = f;
+        }
+      }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  for (int s = 0; s < OP_STAGES - 1; ++s) load_chunk(s);
+  for (int c = 0; c < nch; ++c) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(OP_STAGES - 2) : "memory");
+    __syncthreads();                                    // chunk c is there, chunk c - 1 has been read
+    load_chunk(c + OP_STAGES - 1);
+    if (mine) {
+      const float* xs = rm_smem + (c % OP_STAGES) * ng * OP_GROUP;
+      const float *xr = xs + row(RA * ti), *yr = xs + row(CB * tj);
+#pragma unroll(RA == 8 ? 1 : 8 / RA)
+      for (int k = 0; k < OP_CH; k += 4) {
+        float4 y[CB];
+#pragma unroll
+        for (int q = 0; q < CB; ++q) y[q] = *reinterpret_cast<const float4*>(yr + q * OP_CH + k);
+#pragma unroll
+        for (int a = 0; a < RA; ++a) {
+          const float4 x = *reinterpret_cast<const float4*>(xr + (a >> 2) * OP_GROUP + (a & 3) * OP_CH + k);
+#pragma unroll
+          for (int q = 0; q < CB; ++q) {
+            float v = acc[a][q];
+            v = pair_op<METRIC>(x.x, y[q].x, v);
+            v = pair_op<METRIC>(x.y, y[q].y, v);
+            v = pair_op<METRIC>(x.z, y[q].z, v);
+            v = pair_op<METRIC>(x.w, y[q].w, v);
+            acc[a][q] = v;
+          }
+        }
+      }
+    }
+  }
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  __syncthreads();
+  // the matrix takes the ring's place: rows of T | 1 floats, then the norms
+  const int ld = T | 1;
+  float* norm = rm_smem + T * ld;
+  if (mine) {
+#pragma unroll
+    for (int a = 0; a < RA; ++a)
+#pragma unroll
+      for (int c = 0; c < CB; ++c) {
+        const int t = RA * ti + a, t2 = CB * tj + c;
+        if (t < T && t2 < T) {
+          rm_smem[t * ld + t2] = acc[a][c];
+          rm_smem[t2 * ld + t] = acc[a][c];             // (within the diagonal tiles: the same value twice)
+        }
+      }
+  }
+  __syncthreads();
+  if (METRIC == M_COS) {
+    for (int t = threadIdx.x; t < T; t += blockDim.x) norm[t] = sqrtf(rm_smem[t * ld + t]);
+    __syncthreads();
+  }
+  for (int i = threadIdx.x; i < T * T; i += blockDim.x) {
+    const int t = i / T, t2 = i - t * T;
+    float* g = rm_smem + t * ld + t2;
+    if (METRIC == M_COS) {
+      const float nn = norm[t] * norm[t2];
+      *g = nn == 0.f ? 1.f : 1.f - *g / nn;
+    } else {
+      *g = *g / (float)n;
+    }
+  }
+  __syncthreads();
+  for (int t = threadIdx.x; t < T; t += blockDim.x) {
+    float s = 0.f;
+    for (int t2 = 0; t2 < T; ++t2)
+      if (t2 != t) s += rm_smem[t * ld + t2];
+    dr[((long long)b * N + r) * T + t] = s / (float)(T - 1);
+  }
 }
 
 // d[b][t] = mean over r of dr[b][r][t], summed in order r = 0..N-1
@@ -494,10 +605,10 @@ __global__ void __launch_bounds__(GS_THREADS) guided_kernel(const float* d, int 
   for (int i = threadIdx.x; i < cells; i += GS_THREADS) S[(long long)p * cells + i] = taken[i];
 }
 
-template <int METRIC, int CH>
-cudaError_t launch_pair_ch(const float* rows, int T, int U, int N, int n, int CL, float* dr, cudaStream_t st) {
+template <int CH>
+cudaError_t launch_sorted_pair(const float* rows, int T, int U, int N, int n, int CL, float* dr, cudaStream_t st) {
   const int sm = (int)pair_smem(T);
-  const cudaError_t e = cudaFuncSetAttribute(pair_kernel<METRIC, CH>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  const cudaError_t e = cudaFuncSetAttribute(sorted_pair_kernel<CH>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)pair_smem(CH == 64 ? RM_MAX_T : 32));
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
@@ -512,13 +623,24 @@ cudaError_t launch_pair_ch(const float* rows, int T, int U, int N, int n, int CL
   cfg.stream = st;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, pair_kernel<METRIC, CH>, rows, T, U, N, n, CL, dr);
+  return cudaLaunchKernelEx(&cfg, sorted_pair_kernel<CH>, rows, T, U, N, n, CL, dr);
+}
+
+template <int METRIC, int RA, int CB>
+cudaError_t launch_ordered_pair_as(const float* rows, int T, int U, int N, int n, float* dr, cudaStream_t st) {
+  const cudaError_t e = cudaFuncSetAttribute(ordered_pair_kernel<METRIC, RA, CB>,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)op_smem(RM_MAX_T));
+  if (e != cudaSuccess) return e;
+  const int threads = (op_tiles(T, RA, CB) + 31) / 32 * 32;
+  ordered_pair_kernel<METRIC, RA, CB><<<U * N, threads, op_smem(T), st>>>(rows, T, U, N, n, dr);
+  return cudaGetLastError();
 }
 
 template <int METRIC>
-cudaError_t launch_pair(const float* rows, int T, int U, int N, int n, int CL, float* dr, cudaStream_t st) {
-  return pair_chunk(T) == 64 ? launch_pair_ch<METRIC, 64>(rows, T, U, N, n, CL, dr, st)
-                             : launch_pair_ch<METRIC, 256>(rows, T, U, N, n, CL, dr, st);
+cudaError_t launch_ordered_pair(const float* rows, int T, int U, int N, int n, float* dr, cudaStream_t st) {
+  return T > OP_MID_T     ? launch_ordered_pair_as<METRIC, 8, 4>(rows, T, U, N, n, dr, st)
+         : T > OP_SMALL_T ? launch_ordered_pair_as<METRIC, 4, 2>(rows, T, U, N, n, dr, st)
+                          : launch_ordered_pair_as<METRIC, 2, 2>(rows, T, U, N, n, dr, st);
 }
 
 }  // namespace
@@ -556,18 +678,19 @@ cudaError_t launch_redundancy(const float* trace, int T, int U, int N, int n, in
     if (e != cudaSuccess) return e;
     rows = sorted;
   }
-  // blocks per (b, r): enough for several rounds over the chip's 304 resident
-  // blocks (an even last round), at least four chunks each: 6 units x 1 sample of
-  // 404 entries 46 us, and 83 us undivided; 25 steps x 15 x 7 of 3,516 entries
-  // 52 us, and 43 us with at least eight chunks
+  // sorted rows: blocks per (b, r), enough for several rounds over the chip's
+  // 304 resident blocks (an even last round), at least four chunks each
   int CL = 1;
   const int nch = (n + pair_chunk(T) - 1) / pair_chunk(T);
   while (CL < 8 && (long long)U * N * CL < 1216 && nch >= 4 * CL) CL *= 2;
   cudaError_t e = cudaSuccess;
   switch (metric) {
-    case M_COS: e = launch_pair<M_COS>(rows, T, U, N, n, CL, dr, st); break;
-    case M_MSE: e = launch_pair<M_MSE>(rows, T, U, N, n, CL, dr, st); break;
-    default: e = launch_pair<M_L1>(rows, T, U, N, n, CL, dr, st); break;
+    case M_COS: e = launch_ordered_pair<M_COS>(rows, T, U, N, n, dr, st); break;
+    case M_MSE: e = launch_ordered_pair<M_MSE>(rows, T, U, N, n, dr, st); break;
+    case M_L1: e = launch_ordered_pair<M_L1>(rows, T, U, N, n, dr, st); break;
+    default:
+      e = pair_chunk(T) == 64 ? launch_sorted_pair<64>(rows, T, U, N, n, CL, dr, st)
+                              : launch_sorted_pair<256>(rows, T, U, N, n, CL, dr, st);
   }
   if (e != cudaSuccess) return e;
   mean_kernel<<<(U * T + 255) / 256, 256, 0, st>>>(dr, T, U, N, d);
