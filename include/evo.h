@@ -77,8 +77,11 @@ typedef struct evo_config {
   int32_t job_samples;  /* samples per job (rows = job_samples * horizon); 0 = choose */
   int32_t debug_sync;   /* 1: synchronize after each call and return the device status */
   int32_t wide_rows;    /* batch-wide tensor-core path for calls of at least this many action-token
-                           rows (samples x horizon); 0 = 1024; < 0 = never.  bf16 with n_emb 256 or
-                           512, head size 64, horizon 16 or 32, action dim <= 16, at most 7
+                           rows (samples x horizon); 0 = the library's choice (2048 with a 4-CTA
+                           decomposition, else 1024; and, with cluster and job_samples left to it
+                           too, blocks of 8 samples on their own for calls of 109 samples and more
+                           of n_emb 256, 4 heads, horizon 16); < 0 = never.  bf16 with n_emb 256
+                           or 512, head size 64, horizon 16 or 32, action dim <= 16, at most 7
                            observation tokens */
 } evo_config;
 
@@ -185,7 +188,8 @@ evo_status evo_set_profile_events(evo_handle* h, void* start, void* stop);
  * device array of 8 MiB that every GPU which loads this library holds until
  * the process exits; N * n_obs * (2 * n_layer + 6) * n_emb * 4 bytes must fit
  * in it (186 samples of the Push-T-shaped model), else EVO_ERR_SHAPE and
- * nothing is launched.  No cudaMalloc, cudaFree or allocating library routine
+ * nothing is launched.  (A call that runs on the tile kernel, see wide_rows,
+ * keeps them in the handle's buffers instead; the limit is the same.)  No cudaMalloc, cudaFree or allocating library routine
  * is called.  The first call on a device looks up the array's device address
  * (cudaGetSymbolAddress) and keeps it for later calls.  All calls share the
  * array and every call overwrites all of it
@@ -236,7 +240,9 @@ evo_status evo_get_launch_info(const evo_handle* h, int32_t* cluster, int32_t* j
                                int32_t* max_clusters, int32_t* smem_bytes);
 
 /* How the handle's last call ran: path 0 = one cluster per job (the persistent
- * denoising-loop kernel), 1 = batch-wide (step-synchronous over all samples,
+ * denoising-loop kernel; evo_get_launch_info then says whether a cluster of
+ * several CTAs or, as cluster 1 with 8 samples, a block of the tile kernel),
+ * 1 = batch-wide (step-synchronous over all samples,
  * tensor-core GEMMs); kernels = kernel launches of that call. */
 evo_status evo_get_last_call(const evo_handle* h, int32_t* path, int64_t* kernels);
 

@@ -69,6 +69,9 @@ struct evo_handle {
   // batch-wide path (null when the configuration has none)
   WideState* wide = nullptr;
   long long wide_rows = 1024;
+  // tile path (null when the configuration has none or fixes its decomposition)
+  TileState* tile = nullptr;
+  JobParams tile_base{};              // what evo_get_launch_info reports of it
   int last_path = 0;
   long long last_kernels = 0;
   int last_cond_kernels = 4;          // kernels of the last call's condition path
@@ -84,6 +87,7 @@ struct evo_handle {
   int n_alt = 0;
   const JobParams* last_base = nullptr;   // decomposition of the last cluster launch
   JobParams replan{};                     // a population call's plan with fewer samples per job
+  int *count = nullptr, *order = nullptr; // launch_order
   int last_mc = 0;
 };
 
@@ -466,6 +470,7 @@ evo_status evo_get_launch_info(const evo_handle* h, int32_t* cluster, int32_t* j
 evo_status evo_destroy(evo_handle* h) {
   if (!h) return EVO_ERR_ARG;
   wide_destroy(h->wide);
+  tile_destroy(h->tile);
   cudaFree(h->wf32);
   cudaFree(h->woff_d);
   cudaFree(h->wpack);
@@ -486,6 +491,8 @@ evo_status evo_destroy(evo_handle* h) {
   cudaFree(h->pop_x);
   if (h->stage) cudaFreeHost(h->stage);
   if (h->stage_ev) cudaEventDestroy(h->stage_ev);
+  cudaFree(h->count);
+  cudaFree(h->order);
   delete h;
   return EVO_OK;
 }
@@ -770,11 +777,23 @@ evo_status evo_create(const float* weights, size_t n_floats, const evo_config* c
   if (cudaMalloc(&h->pop_x, cap_samples * H * A * 4) != cudaSuccess) return fail(EVO_ERR_OOM);
   if (cudaMallocHost(&h->stage, h->sched_cap) != cudaSuccess) return fail(EVO_ERR_OOM);
   if (cudaEventCreateWithFlags(&h->stage_ev, cudaEventDisableTiming) != cudaSuccess) return fail(EVO_ERR_CUDA);
+  if (cudaMalloc(&h->count, ((size_t)max_batch + 1) * sizeof(int)) != cudaSuccess ||
+      cudaMalloc(&h->order, ((size_t)max_batch + 1) * sizeof(int)) != cudaSuccess)
+    return fail(EVO_ERR_OOM);
   if (cfg->wide_rows >= 0 && wide_supported(cfg)) {
     // every call's rows (population: (P+1) * N_obs samples) and lattices fit
     const int ws = wide_create(&h->wide, cfg, weights, h->wf32, h->woff, (long long)max_batch * H, max_batch + 1);
     if (ws == EVO_ERR_OOM || ws == EVO_ERR_CUDA) return fail((evo_status)ws);
     if (cfg->wide_rows > 0) h->wide_rows = cfg->wide_rows;
+    // the path is the library's choice: no decomposition or batch-wide threshold is asked for
+    if (ws == EVO_OK && cfg->wide_rows == 0 && cfg->cluster == 0 && cfg->job_samples <= 0 && tile_supported(cfg)) {
+      int ts = tile_create(&h->tile, cfg, weights, h->woff, max_batch);
+      if (ts == EVO_OK) ts = wide_tile_kv(h->wide, weights, h->kv_time);
+      if (ts != EVO_OK) return fail((evo_status)ts);
+      h->tile_base.C = 1;
+      h->tile_base.g = 8;
+      h->tile_base.sm.total = tile_smem_bytes();
+    }
   }
   if (cudaDeviceSynchronize() != cudaSuccess) return fail(EVO_ERR_CUDA);
 
@@ -962,12 +981,88 @@ bool use_wide(const evo_handle* h, long long samples) {
   return h->wide && samples * h->H >= h->wide_rows && samples * h->H <= wide_rows_capacity(h->wide);
 }
 
+// The tile path serves calls of more than three rounds of the 4-CTA clusters
+// (36 fit): 112 samples of the 10-action policy at refresh fraction 0.125 / 1.0
+// take 7.6 / 38.9 ms, four cluster rounds 9.4 / 45.6.
+constexpr long long TILE_MIN_SAMPLES = 109;
+bool use_tile(const evo_handle* h, long long samples) { return h->tile && samples >= TILE_MIN_SAMPLES; }
+
+// Where the batch-wide path is the other choice, it stays ahead on one sparse
+// lattice for few samples (a tile adds the skipped units' caches 64 KiB at a
+// time on one SM): 128 / 208 / 256 samples at fraction 0.05 take 3.5 / 4.0 / 4.8
+// ms there and 4.2 / 4.3 / 4.3 on tiles, at 0.125 7.6 / 8.8 / 10.1 and 7.6.
+bool sparse_for_tile(const evo_handle* h, long long samples, int S_rows) {
+  if (samples >= 224 || samples * h->H < h->wide_rows) return false;
+  const size_t n = (size_t)S_rows * h->T;
+  size_t cells = 0;
+  for (size_t i = 0; i < n; ++i) cells += h->last_sched[i];
+  return 8 * cells < n;
+}
+
+// Lattices for a tile-path call.  Calls of wide_rows rows and more are the ones
+// whose device lattices are checked before anything is launched.
+evo_status stage_tile(evo_handle* h, const uint8_t* S, int n_sched, int rows, bool add_ones, long long samples,
+                      cudaStream_t st, const int** err) {
+  *err = nullptr;
+  if (samples * h->H >= h->wide_rows) return stage_wide(h, S, n_sched, rows, add_ones, st);
+  return stage_schedules(h, S, n_sched, rows, add_ones, st, err);
+}
+
+// The tile path over n_sched staged lattices of N samples each.  More than one
+// lattice: out holds the samples of all, the last is a population's reference
+// (actions: the candidates' copy or null, dev: their deviation).
+evo_status run_tile(evo_handle* h, const float* obs, const float* noise, float* out, int N, int n_sched, int S_rows,
+                    const int* err, cudaStream_t st, float* actions = nullptr, float* dev = nullptr) {
+  long long n = 0;
+  EVO_CUDA(wide_condition(h->wide, obs, N, nullptr, true, h->status, true, st, &n));
+  TileCall c{};
+  EVO_CUDA(wide_masks(h->wide, h->sched, S_rows, n_sched, st, &c.mask));
+  n += 2 + (err ? 1 : 0);
+  if (n_sched > 1) {                           // the longest jobs first
+    EVO_CUDA(launch_order(h->sched, (long long)S_rows * h->T, n_sched, h->count, h->order, st));
+    c.order = h->order;
+    n += 2;
+  }
+  c.noise = noise;
+  c.kv_obs = wide_tile_kv_obs(h->wide);
+  c.kv_time = wide_tile_kv_time(h->wide);
+  c.stab = h->stab;
+  c.out = out;
+  c.sched_err = err;
+  c.n_sched = n_sched;
+  c.per_sched = N;
+  c.obs_mod = N;
+  c.status = h->status;
+  c.st = st;
+  if (h->prof_start && h->prof_stop) EVO_CUDA(cudaEventRecord(h->prof_start, st));
+  EVO_CUDA(tile_run(h->tile, c));
+  if (h->prof_start && h->prof_stop) EVO_CUDA(cudaEventRecord(h->prof_stop, st));
+  const int P = n_sched - 1, HA = h->H * h->A;
+  if (dev) {
+    EVO_CUDA(launch_pop_dev(out, P, N, HA, dev, st));
+    ++n;
+  }
+  if (actions)
+    EVO_CUDA(cudaMemcpyAsync(actions, out, (size_t)P * N * HA * 4, cudaMemcpyDeviceToDevice, st));
+  h->last_base = &h->tile_base;
+  h->last_mc = n_sched * ((N + 7) / 8);
+  h->last_path = 0;
+  h->last_kernels = n;
+  return finish(h, st);
+}
+
 evo_status run(evo_handle* h, const float* obs, const float* noise, const uint8_t* S, int S_rows, int N, float* out,
                float* trace, void* stream) {
   if (!h || !obs || !noise || !S || !out) return EVO_ERR_ARG;
   if (N <= 0 || N > h->max_batch) return EVO_ERR_SHAPE;
   if (S_rows != h->U && S_rows != h->L) return EVO_ERR_SCHEDULE;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+  if (!trace && use_tile(h, N)) {
+    const int* err = nullptr;
+    const evo_status s = stage_tile(h, S, 1, S_rows, false, N, st, &err);
+    if (s != EVO_OK) return s;
+    if (!sparse_for_tile(h, N, S_rows)) return run_tile(h, obs, noise, out, N, 1, S_rows, err, st);
+  }
   if (use_wide(h, N)) {
     const evo_status s = stage_wide(h, S, 1, S_rows, false, st);
     if (s != EVO_OK) return s;
@@ -1062,6 +1157,7 @@ evo_status evo_denoise_noalloc(evo_handle* h, const float* obs, const float* noi
   const int* err = nullptr;
   evo_status s = stage_schedules(h, S, 1, S_rows, false, st, &err);
   if (s != EVO_OK) return s;
+  if (use_tile(h, N)) return run_tile(h, obs, noise, out_actions, N, 1, S_rows, err, st);
   EVO_CUDA(obs_cond(h, obs, N, kv + kv_floats, kv, st));
   const Pick pk = pick_decomposition(h, N);
   JobParams p = *pk.base;
@@ -1092,6 +1188,12 @@ evo_status evo_denoise_population(evo_handle* h, const float* obs, const float* 
   if (S_rows != h->U && S_rows != h->L) return EVO_ERR_SCHEDULE;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   const int HA = h->H * h->A;
+  if (use_tile(h, samples)) {
+    const int* err = nullptr;
+    const evo_status s = stage_tile(h, S_pop, P, S_rows, true, samples, st, &err);
+    if (s != EVO_OK) return s;
+    return run_tile(h, obs, noise, h->pop_x, N_obs, P + 1, S_rows, err, st, out_actions, dev_l2);
+  }
   if (use_wide(h, samples)) {
     const evo_status s = stage_wide(h, S_pop, P, S_rows, true, st);
     if (s != EVO_OK) return s;
@@ -1154,6 +1256,7 @@ evo_status evo_check_guards(evo_handle* h) {
   if (cudaStreamSynchronize(h->last_stream) != cudaSuccess) return EVO_ERR_CUDA;
   int r = guards_check(h->guards);
   if (r == 0 && h->wide) r = guards_check(*wide_guards(h->wide));
+  if (r == 0 && h->tile) r = guards_check(*tile_guards(h->tile));
   return r == 0 ? EVO_OK : (r > 0 ? EVO_ERR_CORRUPT : EVO_ERR_CUDA);
 }
 

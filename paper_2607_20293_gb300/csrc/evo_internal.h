@@ -263,6 +263,8 @@ cudaError_t launch_obs_cond_fast(const float* wf32, const int* woff, const __nv_
                                  float* part, unsigned* count, float* kv_obs, cudaStream_t s);
 cudaError_t launch_obs_cond(const float* wf32, const int* woff_dev, const int* woff, const float* obs, int N,
                             int n_obs, int D, int L, int E, float* scratch, float* kv_obs, cudaStream_t s);
+// lattices [n][bytes] (a uint8 cell each) -> count[n] refreshed cells, order[n] = the lattices by falling count
+cudaError_t launch_order(const uint8_t* S, long long bytes, int n, int* count, int* order, cudaStream_t s);
 cudaError_t launch_validate(const uint8_t* S, long long n, int* err, cudaStream_t s);
 // one CTA, no cluster, no copies: waits on an mbarrier nothing arrives at through
 // the loop kernel's helper (helper 0, limit in cycles) or the tensor-core
@@ -296,6 +298,40 @@ long long wide_rows_capacity(const WideState* w);
 const GuardList* wide_guards(const WideState* w);
 long long wide_last_launches(const WideState* w);
 cudaError_t wide_run(WideState* w, const WideCall& c);
+
+// the steps of a batch-wide call that the tile path shares: the observation
+// tokens' keys/values (to kv_obs unless null; tile: to the tile path's bf16
+// copy; *launches += the kernels launched) and the lattices'
+// per-step bitmasks [n_sched][T][2] (units refreshed, units whose cache holds a value)
+cudaError_t wide_condition(WideState* w, const float* obs, int n, float* kv_obs, bool tile, int* status, bool pdl,
+                           cudaStream_t st, long long* launches);
+cudaError_t wide_masks(WideState* w, const uint8_t* S_dev, int S_rows, int n_sched, cudaStream_t st,
+                       const uint64_t** mask);
+// the tile path's keys/values: weights and buffers, the timestep tokens' copy (from kv_time, fp32 on the device)
+int wide_tile_kv(WideState* w, const float* weights, const float* kv_time);   // evo_status
+const __nv_bfloat16* wide_tile_kv_obs(const WideState* w);
+const __nv_bfloat16* wide_tile_kv_time(const WideState* w);
+
+// tile path (evo_tile.cu): a block per job of up to 8 samples of one lattice
+struct TileState;
+struct TileCall {
+  const float *noise, *stab;
+  const __nv_bfloat16 *kv_obs, *kv_time;   // [obs_mod][n_obs][L][2E], [T][L][2E], head dims in tile_kv_column order
+  float* out;                     // [n_sched * per_sched][H][A]
+  const uint64_t* mask;           // wide_masks
+  const int* sched_err;           // or null; nonzero: the kernel does nothing
+  const int* order;               // or null: the order in which the lattices are taken
+  int n_sched, per_sched, obs_mod;
+  int* status;
+  cudaStream_t st;
+};
+bool tile_supported(const evo_config* c);
+int tile_smem_bytes();
+int tile_kv_column(int part, int p);
+int tile_create(TileState** out, const evo_config* c, const float* weights, const int* woff, int max_batch);   // evo_status
+void tile_destroy(TileState* s);
+const GuardList* tile_guards(const TileState* s);
+cudaError_t tile_run(const TileState* s, const TileCall& c);
 
 // redundancy map and guided sampling (evo_redundancy.cu)
 size_t redundancy_scratch_bytes(int T, int U, int N, int n, int metric);

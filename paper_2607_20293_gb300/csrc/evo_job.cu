@@ -508,6 +508,37 @@ cudaError_t launch_gelu_probe(const float* x, float* y, long long n, int packed,
   return cudaGetLastError();
 }
 
+// a block per lattice: its refreshed cells
+__global__ void count_kernel(const uint8_t* S, long long bytes, int* count) {
+  const uint8_t* s = S + blockIdx.x * bytes;
+  int n = 0;
+  for (long long i = threadIdx.x; i < bytes; i += blockDim.x) n += s[i] != 0;
+  for (int o = 16; o > 0; o >>= 1) n += __shfl_xor_sync(0xffffffffu, n, o);
+  __shared__ int part[8];
+  if (!(threadIdx.x & 31)) part[threadIdx.x >> 5] = n;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < (int)blockDim.x / 32; ++w) n += part[w];
+    count[blockIdx.x] = n;
+  }
+}
+
+// order[rank] = lattice, by falling count (ties by index)
+__global__ void rank_kernel(const int* count, int n, int* order) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const int c = count[i];
+  int r = 0;
+  for (int k = 0; k < n; ++k) r += count[k] > c || (count[k] == c && k < i);
+  order[r] = i;
+}
+
+cudaError_t launch_order(const uint8_t* S, long long bytes, int n, int* count, int* order, cudaStream_t s) {
+  count_kernel<<<n, 256, 0, s>>>(S, bytes, count);
+  rank_kernel<<<(n + 127) / 128, 128, 0, s>>>(count, n, order);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_validate(const uint8_t* S, long long n, int* err, cudaStream_t s) {
   validate_kernel<<<1, 256, 0, s>>>(S, n, err);
   return cudaGetLastError();

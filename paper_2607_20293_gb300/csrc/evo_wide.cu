@@ -764,6 +764,12 @@ struct WideState {
   CUtensorMap mC_qkv, mC_q, mC_hid, mC_cx, mC_ch, mC_cm;
   CUtensorMap mC_r;                 // fp32 r (rbuf), 32 x 32 boxes: the residual GEMM's bulk stores
   BMaps mB_obs, mB_cw1, mB_cw2, mB_kv;
+  // the tile path's keys/values (wide_tile_kv): W_kv^T and bias with the head dims reordered,
+  // the timestep tokens' [T][L][2E], the observation tokens' [tokcap][L][2E]
+  __nv_bfloat16 *tkv_w = nullptr, *tkv_time = nullptr, *tkv_obs = nullptr;
+  float* tkv_b = nullptr;
+  BMaps mB_tkv;
+  CUtensorMap mC_tkv;
   int num_sms = 0;
   GuardList guards;                 // guard bands of the activation buffers
   // replay of a repeated call's launch sequence (wide_run)
@@ -1067,6 +1073,10 @@ void wide_destroy(WideState* w) {
   cudaFree(w->cm16);
   cudaFree(w->cw_t);
   cudaFree(w->bkv);
+  cudaFree(w->tkv_w);
+  cudaFree(w->tkv_b);
+  cudaFree(w->tkv_time);
+  cudaFree(w->tkv_obs);
   if (w->exec) cudaGraphExecDestroy(w->exec);
   if (w->cap_stream) cudaStreamDestroy(w->cap_stream);
   delete w;
@@ -1075,6 +1085,109 @@ void wide_destroy(WideState* w) {
 long long wide_rows_capacity(const WideState* w) { return w ? w->rmax : 0; }
 const GuardList* wide_guards(const WideState* w) { return &w->guards; }
 long long wide_last_launches(const WideState* w) { return w ? w->launches : 0; }
+
+// Observation tokens of n samples -> keys/values: a chain of five or six kernels.
+cudaError_t wide_condition(WideState* w, const float* obs, int n, float* kv_obs, bool tile, int* status, bool pdl,
+                           cudaStream_t st, long long* launches) {
+  const int E = w->E, L = w->L;
+  cudaError_t e;
+#define WCK(x)                    \
+  do {                            \
+    e = (x);                      \
+    if (e != cudaSuccess) return e; \
+    ++*launches;                  \
+  } while (0)
+  // observation tokens -> their cross-attention keys/values of every layer:
+  // bf16 features, embedding (+ b_obs + position row), MLP E -> 4E (Mish) -> E,
+  // then one GEMM for the keys|values of all layers (fp32 out)
+  const int ntok = n * w->n_obs;
+  const int tp = (ntok + tc::BM - 1) / tc::BM * tc::BM;
+  const long long nel = (long long)ntok * w->Dp;
+  WCK(launch_pdl(pdl, obs_to_bf16_kernel, dim3((unsigned)std::min<long long>((nel + 255) / 256, 4096)), dim3(256), 0,
+                 st, obs, ntok, w->D, w->Dp, w->obs16));
+  tc::GemmArgs q{};
+  q.rows = ntok;
+  q.status = status;
+  q.wait_limit = WAIT_POLLS_DEFAULT;
+  q.K = w->Dp;
+  q.bias = w->wf32 + w->woff[W_OBS_B];
+  q.rbias = w->wf32 + w->woff[W_COND_POS] + E;      // position rows 1 .. n_obs
+  q.rbias_mod = w->n_obs;
+  q.out = w->cx16;
+  q.ldo = E;
+  WCK(gemm<tc::EPI_BF16>(w->mA_obs, w->mB_obs, w->mC_cx, q, tp, E, w->num_sms, pdl, st));
+  q.rbias = nullptr;
+  q.K = E;
+  q.bias = w->wf32 + w->woff[W_CM_B1];
+  q.out = w->ch16;
+  q.ldo = 4 * E;
+  WCK(gemm<tc::EPI_MISH_BF16>(w->mA_cx, w->mB_cw1, w->mC_ch, q, tp, 4 * E, w->num_sms, pdl, st));
+  q.K = 4 * E;
+  q.bias = w->wf32 + w->woff[W_CM_B2];
+  q.out = w->cm16;
+  q.ldo = E;
+  WCK(gemm<tc::EPI_BF16>(w->mA_ch, w->mB_cw2, w->mC_cm, q, tp, E, w->num_sms, pdl, st));
+  q.K = E;
+  q.ldo = L * 2 * E;
+  if (kv_obs) {
+    q.bias = w->bkv;
+    q.out32 = kv_obs;
+    WCK(gemm<tc::EPI_F32>(w->mA_cm, w->mB_kv, w->mC_cm, q, tp, L * 2 * E, w->num_sms, pdl, st));
+  }
+  if (tile) {
+    q.bias = w->tkv_b;
+    q.out = w->tkv_obs;
+    WCK(gemm<tc::EPI_BF16>(w->mA_cm, w->mB_tkv, w->mC_tkv, q, tp, L * 2 * E, w->num_sms, pdl, st));
+  }
+#undef WCK
+  return cudaSuccess;
+}
+
+cudaError_t wide_masks(WideState* w, const uint8_t* S_dev, int S_rows, int n_sched, cudaStream_t st,
+                       const uint64_t** mask) {
+  if (n_sched > w->max_sched) return cudaErrorInvalidValue;
+  Lat lat{};
+  lat.S = S_dev;
+  lat.stride = (long long)S_rows * w->T;
+  lat.S_rows = S_rows;
+  lat.U = w->U;
+  lat.T = w->T;
+  lat.force = w->force;
+  *mask = w->mask;
+  return launch_pdl(false, first_kernel, dim3(n_sched), dim3(64), 0, st, lat, n_sched, w->first, w->mask);
+}
+
+int wide_tile_kv(WideState* w, const float* weights, const float* kv_time) {
+  const int E = w->E, L = w->L, KV = L * 2 * E;
+  const size_t nt = (size_t)w->T * KV;
+  // column j of a layer's keys | values -> the column of W_kv that stands there
+  std::vector<int> col(2 * E);
+  for (int j = 0; j < 2 * E; ++j) col[j] = j / 64 * 64 + tile_kv_column(j / E, j % 64);
+  std::vector<uint16_t> wt((size_t)KV * E), tt(nt);
+  std::vector<float> bias(KV), tf(nt);
+  for (int l = 0; l < L; ++l) {
+    const float* base = weights + w->woff[W_LAYER0] + (size_t)l * w->woff[W_LAYER_STRIDE];
+    const float *wkv = base + w->woff[WL_CA_WKV], *bkv = base + w->woff[WL_CA_BKV];
+    for (int j = 0; j < 2 * E; ++j) {
+      for (int k = 0; k < E; ++k) wt[((size_t)l * 2 * E + j) * E + k] = bf16_bits(wkv[(size_t)k * 2 * E + col[j]]);
+      bias[(size_t)l * 2 * E + j] = bkv[col[j]];
+    }
+  }
+  if (cudaMemcpy(tf.data(), kv_time, nt * 4, cudaMemcpyDeviceToHost) != cudaSuccess) return EVO_ERR_CUDA;
+  for (size_t i = 0; i < nt; ++i) tt[i] = bf16_bits(tf[i / (2 * E) * (2 * E) + col[i % (2 * E)]]);
+  if (cudaMalloc(&w->tkv_w, wt.size() * 2) != cudaSuccess || cudaMalloc(&w->tkv_b, bias.size() * 4) != cudaSuccess ||
+      cudaMalloc(&w->tkv_time, nt * 2) != cudaSuccess || cudaMalloc(&w->tkv_obs, w->tokcap * KV * 2) != cudaSuccess)
+    return EVO_ERR_OOM;
+  if (cudaMemcpy(w->tkv_w, wt.data(), wt.size() * 2, cudaMemcpyHostToDevice) != cudaSuccess ||
+      cudaMemcpy(w->tkv_b, bias.data(), bias.size() * 4, cudaMemcpyHostToDevice) != cudaSuccess ||
+      cudaMemcpy(w->tkv_time, tt.data(), nt * 2, cudaMemcpyHostToDevice) != cudaSuccess ||
+      !make_map(&w->mB_tkv.n128, w->tkv_w, KV, E, 128) || !make_map(&w->mB_tkv.n256, w->tkv_w, KV, E, 256) ||
+      !make_map(&w->mC_tkv, w->tkv_obs, w->tokcap, KV, 32))
+    return EVO_ERR_CUDA;
+  return EVO_OK;
+}
+const __nv_bfloat16* wide_tile_kv_obs(const WideState* w) { return w->tkv_obs; }
+const __nv_bfloat16* wide_tile_kv_time(const WideState* w) { return w->tkv_time; }
 
 namespace {
 
@@ -1116,43 +1229,7 @@ cudaError_t wide_launch(WideState* w, const WideCall& c, cudaStream_t st) {
   lat.H = H;
   lat.per_sched = c.per_sched;
   lat.force = w->force;
-  if (c.obs) {
-    // observation tokens -> their cross-attention keys/values of every layer:
-    // bf16 features, embedding (+ b_obs + position row), MLP E -> 4E (Mish) -> E,
-    // then one GEMM for the keys|values of all layers (fp32 out)
-    const int ntok = c.obs_mod * w->n_obs;
-    const int tp = (ntok + tc::BM - 1) / tc::BM * tc::BM;
-    const long long nel = (long long)ntok * w->Dp;
-    WCK(launch_pdl(pdl, obs_to_bf16_kernel, dim3((unsigned)std::min<long long>((nel + 255) / 256, 4096)), dim3(256), 0,
-                   st, c.obs, ntok, w->D, w->Dp, w->obs16));
-    tc::GemmArgs q{};
-    q.rows = ntok;
-    q.status = c.status;
-    q.wait_limit = WAIT_POLLS_DEFAULT;
-    q.K = w->Dp;
-    q.bias = w->wf32 + w->woff[W_OBS_B];
-    q.rbias = w->wf32 + w->woff[W_COND_POS] + E;      // position rows 1 .. n_obs
-    q.rbias_mod = w->n_obs;
-    q.out = w->cx16;
-    q.ldo = E;
-    WCK(gemm<tc::EPI_BF16>(w->mA_obs, w->mB_obs, w->mC_cx, q, tp, E, w->num_sms, pdl, st));
-    q.rbias = nullptr;
-    q.K = E;
-    q.bias = w->wf32 + w->woff[W_CM_B1];
-    q.out = w->ch16;
-    q.ldo = 4 * E;
-    WCK(gemm<tc::EPI_MISH_BF16>(w->mA_cx, w->mB_cw1, w->mC_ch, q, tp, 4 * E, w->num_sms, pdl, st));
-    q.K = 4 * E;
-    q.bias = w->wf32 + w->woff[W_CM_B2];
-    q.out = w->cm16;
-    q.ldo = E;
-    WCK(gemm<tc::EPI_BF16>(w->mA_ch, w->mB_cw2, w->mC_cm, q, tp, E, w->num_sms, pdl, st));
-    q.K = E;
-    q.bias = w->bkv;
-    q.out32 = c.kv_obs;
-    q.ldo = L * 2 * E;
-    WCK(gemm<tc::EPI_F32>(w->mA_cm, w->mB_kv, w->mC_cm, q, tp, L * 2 * E, w->num_sms, pdl, st));
-  }
+  if (c.obs && (e = wide_condition(w, c.obs, c.obs_mod, c.kv_obs, false, c.status, pdl, st, &n)) != cudaSuccess) return e;
   WCK(launch_pdl(pdl, first_kernel, dim3(c.n_sched), dim3(64), 0, st, lat, c.n_sched, w->first, w->mask));
 
   Walk wp{};

@@ -1,0 +1,118 @@
+"""GPU parity of the tile path (one block runs the whole loop of up to 8 samples)
+against the float64 oracle: the library's own choice from 109 samples on for
+n_emb 256, horizon 16.
+
+Cases are the edges of its tiles and operands: a last tile of 1 .. 8 samples,
+1 and 16 actions, 1 and 7 observation tokens (2 and 8 memory keys), both
+samplers and empty-cache policies, coarse and device lattices, lattices that
+refresh nothing, one cell or everything.  Tolerance: max-abs 3e-2 on final
+actions (bf16 mode), on sampled chunks."""
+import numpy as np
+import pytest
+
+from oracle import evo_oracle as O
+from paper_2607_20293_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+TOL = 3e-2
+
+
+@pytest.fixture(scope="module")
+def torch():
+    import torch as _t
+    if not _t.cuda.is_available():
+        pytest.skip("no CUDA device")
+    return _t
+
+
+@pytest.fixture(scope="module")
+def B(torch):
+    from paper_2607_20293_gb300 import binding, build
+    build.build()
+    binding.load()
+    return binding
+
+
+def on_tiles(ev):
+    info = ev.launch_info()
+    return info["cluster"] == 1 and info["job_samples"] == 8
+
+
+def close(got, want, what=""):
+    assert np.all(np.isfinite(got)), what
+    err = float(np.max(np.abs(got - want)))
+    assert err <= TOL, f"{what}: max-abs {err:.3e}"
+
+
+# 109 = 13 tiles and 5 samples, 112 = 14 full tiles, 113 = a tile of one sample
+@pytest.mark.parametrize("n,over,frac", [
+    (109, {}, 0.3),
+    (112, dict(action_dim=16, n_obs=7, obs_dim=30), 1.0),
+    (113, dict(action_dim=1, n_obs=1), 0.125),
+    (120, dict(sampler="ddim", n_layer=1), 0.5),
+    (230, dict(n_layer=2, action_dim=5), 0.05),
+])
+def test_tile_matches_oracle(torch, B, n, over, frac):
+    cfg = synth.config("pusht", n_steps=20, **over)
+    units = 3 * cfg["n_layer"]
+    W = synth.make_weights(cfg, 0)
+    obs, noise = synth.make_obs(cfg, n, 71), synth.make_noise(cfg, n, 72)
+    S = np.ones((units, 20), np.uint8) if frac == 1.0 else synth.bernoulli_schedule(units, 20, frac, 73)
+    ev = B.Evo(cfg, W, n)
+    got = ev.denoise(torch.from_numpy(obs).cuda(), torch.from_numpy(noise).cuda(), S).cpu().numpy()
+    assert on_tiles(ev)
+    idx = [0, 7, 8, n - 2, n - 1]
+    close(got[idx], O.denoise(W, cfg, obs[idx], noise[:, idx], S), f"n={n}")
+    assert ev.status() == B.OK
+
+
+@pytest.mark.parametrize("empty", ["zero", "force"])
+def test_tile_population_edge_lattices(torch, B, empty):
+    # 11 observations: a tile of 8 samples and one of 3 per lattice
+    cfg = synth.config("pusht", n_steps=20, n_layer=2)
+    U, T, N = 6, 20, 11
+    W = synth.make_weights(cfg, 0)
+    lat = np.zeros((11, U, T), np.uint8)
+    lat[0, 0, 0] = 1                  # the first cell only
+    lat[1, U - 1, T - 1] = 1          # the last cell only
+    lat[2, :, 0] = 1                  # every unit at step 0, then skips to the end
+    lat[3, :, T - 1] = 1
+    lat[4] = 1                        # the reference itself; lattice 5: nothing refreshed
+    for p in range(6, 11):
+        lat[p] = synth.bernoulli_schedule(U, T, 0.1 * p, p)
+    obs, noise = synth.make_obs(cfg, N, 81), synth.make_noise(cfg, N, 82)
+    ev = B.Evo(cfg, W, 12 * N, empty=empty)
+    x, dev = ev.population(torch.from_numpy(obs).cuda(), torch.from_numpy(noise).cuda(), lat)
+    assert on_tiles(ev)
+    x, dev = x.cpu().numpy(), dev.cpu().numpy()
+    idx = [0, 7, 8, 10]
+    for p in range(11):
+        close(x[p][idx], O.denoise(W, cfg, obs[idx], noise[:, idx], lat[p], policy=empty), f"lattice {p} ({empty})")
+    assert dev[4] == 0.0              # the same jobs on the same kernel
+    full = x[4]
+    want = np.linalg.norm((x - full[None]).reshape(11, N, -1), axis=2).mean(1)
+    assert np.allclose(dev, want, rtol=1e-4, atol=1e-5)
+
+
+def test_tile_lattice_forms(torch, B):
+    # coarse [L][T] and device lattices give the bits of the unit lattice on the
+    # host; an invalid device lattice is reported and leaves the output alone
+    cfg = synth.config("pusht", n_steps=20, n_layer=2)
+    n = 110
+    W = synth.make_weights(cfg, 0)
+    obs = torch.from_numpy(synth.make_obs(cfg, n, 91)).cuda()
+    noise = torch.from_numpy(synth.make_noise(cfg, n, 92)).cuda()
+    S = synth.bernoulli_schedule(2, 20, 0.4, 93)
+    ev = B.Evo(cfg, W, n)
+    want = ev.denoise(obs, noise, np.repeat(S, 3, axis=0)).cpu().numpy()
+    assert on_tiles(ev)
+    assert np.array_equal(ev.denoise(obs, noise, S).cpu().numpy(), want)
+    assert np.array_equal(ev.denoise(obs, noise, torch.from_numpy(S).cuda()).cpu().numpy(), want)
+    bad = torch.from_numpy(S).cuda()
+    bad[1, 3] = 2
+    out = torch.full((n, 16, 2), 5.0, device="cuda")
+    ev.denoise(obs, noise, bad, out=out)
+    assert ev.status() == B.ERR_SCHEDULE
+    assert torch.all(out == 5.0)
+    assert np.array_equal(ev.denoise_noalloc(obs, noise, S, out).cpu().numpy(), want)
