@@ -207,6 +207,7 @@ struct JobParams {
   float invE;                     // 1 / E
   int kp_o, kp_h;                 // K of the second GEMMs (attention: Ec, FFN: hid), multiples of 16
   int n_jobs;
+  const int* order;               // or null: cluster i of a cluster-per-job launch takes a job of lattice order[..] (per_sched % g == 0)
   int sampler, force;
   int nslot, slot_bytes;
   long long wait_limit;           // SM cycles before a wait gives up (WAIT_CYCLES_DEFAULT)

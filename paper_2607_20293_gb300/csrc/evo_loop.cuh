@@ -1217,7 +1217,12 @@ __global__ void __launch_bounds__(NTHREADS, 1) job_kernel(const __grid_constant_
       cx.kv_dst = (i * p.Cm + tok) * S::kvw + (w < kq ? 4 * w : S::dh + 4 * (w - kq));
     }
   }
-  const uint32_t cid = cluster_idx(), ncl = cluster_count();
+  uint32_t cid = cluster_idx();
+  const uint32_t ncl = cluster_count();
+  if (p.order) {                                  // a cluster per job, those of the longest lattices first
+    const uint32_t per = (uint32_t)p.per_sched / S::G, k = cid / per;
+    cid = (uint32_t)p.order[k] * per + (cid - k * per);
+  }
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < S::NSLOT; ++i) {
