@@ -48,9 +48,9 @@
 // Bound by instruction issue and its dependent chains on two compute warps per
 // SM sub-partition (the register file holds no more of them beside the stream:
 // with sixteen warps of half a row the compiler spills it).  A unit takes about
-// 16 us.  64 candidates x 16 observations and their reference (n_emb 256, 8
-// layers, 100 steps): 97.5 ms batch-wide -> 38.5 ms, the reference's 2,400
-// units; 300 samples at refresh fraction 0.125: 10.3 -> 7.6 ms.
+// 14 us.  64 candidates x 16 observations and their reference (n_emb 256, 8
+// layers, 100 steps): 97.5 ms batch-wide -> 34.6 ms, the reference's 2,400
+// units; 300 samples at refresh fraction 0.125: 10.3 -> 7.1 ms.
 //
 // Warps 0-7 compute, warp 8 streams weights, warp 9 issues the MMAs (10 and 11
 // only complete the third warpgroup, which gives its registers away).  Every
@@ -128,10 +128,24 @@ struct TileParams {
 
 __device__ __forceinline__ void bar_compute() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
 
-__device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(su32(dst)),
-               "l"(src), "r"(bytes), "r"(su32(bar))
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+               "l"(src), "r"(bytes), "r"(bar)
                : "memory");
+}
+__device__ __forceinline__ void expect_tx(uint32_t bar, uint32_t bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void commit(uint32_t bar) {
+  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ uint64_t desc64(uint32_t lo, uint32_t hi) { return ((uint64_t)hi << 32) | lo; }
+__device__ __noinline__ void wait_slow(uint32_t bar, uint32_t parity, int* status, long long limit) {
+  for (long long i = 0; i < limit; ++i) {
+    if (mbar_test(bar, parity)) return;
+    if (i > 64) __nanosleep(32);
+  }
+  atomicOr(status, ST_TIMEOUT);
 }
 
 // 16 rows x 32 (64) fp32 columns in the layout of mma.sync accumulators: tile j
@@ -162,6 +176,19 @@ __device__ __forceinline__ void tmem_ld_frag(uint32_t taddr, float (&v)[8][4]) {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
   for (int i = 0; i < 32; ++i) v[i >> 2][i & 3] = __uint_as_float(r[i]);
+}
+
+// 16 columns of it, issued ahead: the registers hold them after tmem_wait
+__device__ __forceinline__ void tmem_ld_ahead(uint32_t taddr, uint32_t (&r)[8]) {
+  asm volatile("tcgen05.ld.sync.aligned.16x256b.x2.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr));
+}
+__device__ __forceinline__ void tmem_wait(uint32_t (&r)[8]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7])
+               :
+               : "memory");
 }
 
 __device__ __forceinline__ uint32_t pk2(float x, float y) {
@@ -358,117 +385,136 @@ __global__ void __launch_bounds__(TTHREADS, 1) tile_kernel(const TileParams p) {
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = B->tslot;
-  const uint32_t tR = tmem, tA = tmem + 256;
+  const uint32_t tmem = B->tslot, tR = tmem, tA = tmem + 256;
 
   if (warp >= 8) {
-   asm volatile("setmaxnreg.dec.sync.aligned.u32 104;");
-   if (warp == 8) {
-    // ------------------------------------------------ weights and vectors: bulk copies
-    if (lane == 0) {
-      uint32_t q = 0, units = 0;
-      for (int j = blockIdx.x; j < p.n_jobs; j += gridDim.x) {
-        const int lat = lattice_of(p, j);
-        const uint64_t* mk = p.mask + (long long)lat * p.T * 2;
-        uint64_t nxt = __ldg(mk);
-        for (int t = 0; t < p.T; ++t) {
-          uint64_t m = nxt;
-          if (t + 1 < p.T) nxt = __ldg(mk + 2 * (t + 1));
-          while (m) {
-            const int b = __ffsll((long long)m) - 1, u = b % 3;
-            m &= m - 1;
-            const uint8_t* src = p.wpack + ((long long)(b / 3) * LAYER_SLOTS + unit_slot0(u)) * SLOT;
-            const int ns = unit_slots(u), vb = units & 1;
-            mbar_wait(&B->vempty[vb], ((units >> 1) & 1u) ^ 1u, p.status, p.wait_limit);
-            mbar_expect_tx(&B->vfull[vb], vec_floats(u) * 4);
-            bulk_load(vecs + vb * (VEC_BYTES / 4), p.vec + (long long)(b / 3) * VEC_LAYER + vec_off(u),
-                      vec_floats(u) * 4, &B->vfull[vb]);
-            ++units;
-            for (int i = 0; i < ns; ++i, ++q) {
-              const uint32_t s = q % NSLOTS;
-              mbar_wait(&B->empty[s], ((q / NSLOTS) & 1u) ^ 1u, p.status, p.wait_limit);
-              mbar_expect_tx(&B->full[s], SLOT);
-              bulk_load(ring + s * SLOT, src + (long long)i * SLOT, SLOT, &B->full[s]);
-            }
-          }
-        }
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 104;");
+    // Both walk the refreshed units as the compute warps do.  Their loops set
+    // the pace of the weights (a slot is 256 cycles of MMAs), so they count
+    // slots and phases instead of dividing, work on 32-bit shared addresses and
+    // descriptor words, leave a wait that does not pass at once to a call, and
+    // run uniformly over the warp with one elected lane issuing (1,000 samples at
+    // full refresh: 39.4 ms with one lane in a divergent branch, 35.0).
+    const uint32_t bfull = su32(B->full), bempty = su32(B->empty);
+    uint32_t s = 0, ph = 0;                            // ring slot, its phase
+    auto next_slot = [&]() {
+      if (++s == NSLOTS) {
+        s = 0;
+        ph ^= 1u;
       }
-    }
-  } else if (warp == 9) {
-    // ------------------------------------------------ MMA issue
-    if (lane == 0) {
-      constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(TROWS >> 4) << 24);
-      constexpr uint32_t ID = IDESC | ((128u >> 3) << 17);
-      const uint64_t dx = sw128_desc(su32(xln)), dh = sw128_desc(su32(hid)), dr = sw128_desc(su32(ring));
-      uint32_t q = 0, units = 0;            // slots consumed, refreshed units so far
-      uint32_t na = 0, nh[2] = {0, 0};      // first-GEMM chunks issued; second-GEMM chunks by buffer
-      auto first = [&](int) {
-        const uint32_t acc = na & 1u;
-        mbar_wait(&B->aempty[acc], ((na >> 1) & 1u) ^ 1u, p.status, p.wait_limit);
-        tc_fence_after();
-        const uint32_t d = tA + acc * 128;
-        for (int kb = 0; kb < 4; ++kb, ++q) {
-          const uint32_t s = q % NSLOTS;
-          mbar_wait(&B->full[s], (q / NSLOTS) & 1u, p.status, p.wait_limit);
-          tc_fence_after();
-#pragma unroll
-          for (int k = 0; k < 4; ++k)
-            mma_f16(d, dx + (uint64_t)(kb * (16384 >> 4) + 2 * k), dr + (uint64_t)(s * (SLOT >> 4) + 2 * k), ID,
-                    (kb | k) != 0);
-          mma_commit(&B->empty[s]);
-        }
-        mma_commit(&B->afull[acc]);
-        ++na;
-      };
-      auto second = [&](int c) {
-        const int buf = c & 1;
-        mbar_wait(&B->hready[buf], nh[buf] & 1u, p.status, p.wait_limit);
-        tc_fence_after();
-        for (int i = 0; i < 4; ++i, ++q) {              // K block i / 2, columns 128 (i & 1) ..
-          const uint32_t s = q % NSLOTS;
-          mbar_wait(&B->full[s], (q / NSLOTS) & 1u, p.status, p.wait_limit);
-          tc_fence_after();
-#pragma unroll
-          for (int k = 0; k < 4; ++k)
-            mma_f16(tR + (i & 1) * 128, dh + (uint64_t)(buf * (HID_BYTES >> 4) + (i >> 1) * (16384 >> 4) + 2 * k),
-                    dr + (uint64_t)(s * (SLOT >> 4) + 2 * k), ID, (c | (i >> 1) | k) != 0);
-          mma_commit(&B->empty[s]);
-        }
-        mma_commit(&B->hempty[buf]);
-        ++nh[buf];
-      };
+    };
+    auto wait = [&](uint32_t bar, uint32_t parity) {
+      if (!mbar_test(bar, parity)) wait_slow(bar, parity, p.status, p.wait_limit);
+    };
+    if (warp == 8) {
+      // ------------------------------------------------ weights and vectors: bulk copies
+      const uint32_t bvfull = su32(B->vfull), bvempty = su32(B->vempty), dring = su32(ring), dvec = su32(vecs);
+      uint32_t units = 0;
       for (int j = blockIdx.x; j < p.n_jobs; j += gridDim.x) {
-        const int lat = lattice_of(p, j);
-        const uint64_t* mk = p.mask + (long long)lat * p.T * 2;
+        const uint64_t* mk = p.mask + (long long)lattice_of(p, j) * p.T * 2;
         uint64_t nxt = __ldg(mk);
         for (int t = 0; t < p.T; ++t) {
           uint64_t m = nxt;
           if (t + 1 < p.T) nxt = __ldg(mk + 2 * (t + 1));
           while (m) {
-            const int b = __ffsll((long long)m) - 1, u = b % 3;
+            const int b = __ffsll((long long)m) - 1, l = b / 3, u = b - 3 * l;
             m &= m - 1;
-            mbar_wait(&B->xready, units & 1u, p.status, p.wait_limit);
-            tc_fence_after();
-            // the order in which pack_unit lays out the slots
-            if (u == 2) {
-              first(0);
-              for (int c = 1; c < 8; ++c) {
-                first(c);
-                second(c - 1);
+            const uint32_t vb = units & 1;
+            wait(bvempty + 8 * vb, ((units >> 1) & 1u) ^ 1u);
+            if (elect_one()) {
+              expect_tx(bvfull + 8 * vb, vec_floats(u) * 4);
+              bulk_load(dvec + vb * VEC_BYTES, p.vec + (long long)l * VEC_LAYER + vec_off(u), vec_floats(u) * 4,
+                        bvfull + 8 * vb);
+            }
+            ++units;
+            const uint8_t* src = p.wpack + ((long long)l * LAYER_SLOTS + unit_slot0(u)) * SLOT;
+            const uint8_t* end = src + unit_slots(u) * SLOT;
+#pragma unroll 1
+            for (; src != end; src += SLOT) {
+              wait(bempty + 8 * s, ph ^ 1u);
+              if (elect_one()) {
+                expect_tx(bfull + 8 * s, SLOT);
+                bulk_load(dring + s * SLOT, src, SLOT, bfull + 8 * s);
               }
-              second(7);
-            } else {
-              for (int c = 0; c < n_first(u); ++c) first(c);
-              second(0);
-              second(1);
+              next_slot();
             }
-            mma_commit(&B->rfull);
+          }
+        }
+      }
+    } else if (warp == 9) {
+      // ------------------------------------------------ MMA issue
+      constexpr uint32_t ID = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(TROWS >> 4) << 24) | ((128u >> 3) << 17);
+      const uint64_t d0 = sw128_desc(0);
+      const uint32_t dhi = (uint32_t)(d0 >> 32), dlo = (uint32_t)d0;     // + (address >> 4)
+      const uint32_t dx = dlo + (su32(xln) >> 4), dh = dlo + (su32(hid) >> 4), dr = dlo + (su32(ring) >> 4);
+      const uint32_t baf = su32(B->afull), bae = su32(B->aempty), bhr = su32(B->hready), bhe = su32(B->hempty);
+      const uint32_t bx = su32(&B->xready), brf = su32(&B->rfull);
+      uint32_t units = 0, na = 0, nh = 0;               // phases: units, first-GEMM chunks; second-GEMM chunks / 2
+      for (int j = blockIdx.x; j < p.n_jobs; j += gridDim.x) {
+        const uint64_t* mk = p.mask + (long long)lattice_of(p, j) * p.T * 2;
+        uint64_t nxt = __ldg(mk);
+        for (int t = 0; t < p.T; ++t) {
+          uint64_t m = nxt;
+          if (t + 1 < p.T) nxt = __ldg(mk + 2 * (t + 1));
+          while (m) {
+            const int b = __ffsll((long long)m) - 1, u = b % 3;
+            m &= m - 1;
+            wait(bx, units & 1u);
+            tc_fence_after();
+            const int nf = n_first(u), n_ops = nf + n_second(u);
+            int c2 = 0;                                 // second-GEMM chunk
+            // the order in which pack_unit lays out the slots
+#pragma unroll 1
+            for (int i = 0; i < n_ops; ++i) {
+              const bool first = u == 2 ? i < 3 || ((i & 1) == 0 && i < 14) : i < nf;
+              uint32_t da, d, sa, sd, acc, bdone;       // A, D and their steps per slot
+              if (first) {
+                const uint32_t a = na & 1u;
+                wait(bae + 8 * a, ((na >> 1) & 1u) ^ 1u);
+                da = dx;
+                sa = 0;                                 // K block: the slot
+                d = tA + a * 128;
+                sd = 0;
+                acc = 0;
+                bdone = baf + 8 * a;
+                ++na;
+              } else {
+                const uint32_t buf = c2 & 1u;
+                wait(bhr + 8 * buf, nh & 1u);
+                da = dh + buf * (HID_BYTES >> 4);
+                sa = 1;                                 // K block: the slot / 2, columns 128 (slot & 1)
+                d = tR;
+                sd = 128;
+                acc = c2 > 0;
+                bdone = bhe + 8 * buf;
+                nh += buf;                              // the buffers alternate
+                ++c2;
+              }
+              tc_fence_after();
+#pragma unroll 1
+              for (uint32_t k = 0; k < 4; ++k) {
+                wait(bfull + 8 * s, ph);
+                tc_fence_after();
+                const uint32_t kb = k >> sa, ak = da + kb * (16384 >> 4), bk = dr + s * (SLOT >> 4);
+                const uint32_t dk = d + (k & 1u) * sd;
+                if (elect_one()) {
+#pragma unroll
+                  for (uint32_t e = 0; e < 4; ++e)
+                    mma_f16(dk, desc64(ak + 2 * e, dhi), desc64(bk + 2 * e, dhi), ID, acc | kb | e);
+                  commit(bempty + 8 * s);
+                  if (k == 3) {
+                    commit(bdone);
+                    if (i == n_ops - 1) commit(brf);
+                  }
+                }
+                next_slot();
+              }
+            }
             ++units;
           }
         }
       }
     }
-   }
   } else {
     asm volatile("setmaxnreg.inc.sync.aligned.u32 200;");
     // ------------------------------------------------ compute warps
@@ -617,26 +663,26 @@ __global__ void __launch_bounds__(TTHREADS, 1) tile_kernel(const TileParams p) {
             for (int c = 0; c < 8; ++c) {
               const uint32_t acc = wait_acc();
               const int buf = c & 1;
+              // 16 columns at a time, the next ones on their way: four pairs of
+              // GELUs side by side are what the registers leave room for
+              const uint32_t src = tA + acc * 128 + lanes;
+              const float2* bb = reinterpret_cast<const float2*>(vec + 768 + c * 128) + tq;
+              uint32_t v[2][8];
+              tmem_ld_ahead(src, v[0]);
+              wait_hid(buf);
 #pragma unroll
-              for (int h = 0; h < 2; ++h) {             // 64 columns at a time
-                float v[8][4];
-                tmem_ld_frag(tA + acc * 128 + h * 64 + lanes, v);
-                if (h == 1) free_acc(acc);
-                const float2* bb = reinterpret_cast<const float2*>(vec + 768 + c * 128 + h * 64) + tq;
-                uint32_t pk[16];
-#pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                  const float2 bi = bb[4 * i];
-                  const float2 y0 = gelu_as2(add2(make_float2(v[i][0], v[i][1]), bi));
-                  const float2 y1 = gelu_as2(add2(make_float2(v[i][2], v[i][3]), bi));
-                  pk[2 * i] = pk2(y0.x, y0.y);
-                  pk[2 * i + 1] = pk2(y1.x, y1.y);
-                }
-                if (h == 0) wait_hid(buf);
-#pragma unroll
-                for (int i = 0; i < 8; i += 2)
-                  put_tiles(hid + buf * HID_BYTES + h * 16384, row0, i, lane, pk[2 * i], pk[2 * i + 1], pk[2 * i + 2],
-                            pk[2 * i + 3]);
+              for (int i = 0; i < 8; ++i) {
+                uint32_t(&w)[8] = v[i & 1];
+                tmem_wait(w);
+                if (i < 7) tmem_ld_ahead(src + 16 * (i + 1), v[(i + 1) & 1]);
+                else free_acc(acc);
+                const float2 b0 = bb[8 * i], b1 = bb[8 * i + 4];
+                const float2 y0 = gelu_as2(add2(make_float2(__uint_as_float(w[0]), __uint_as_float(w[1])), b0));
+                const float2 y1 = gelu_as2(add2(make_float2(__uint_as_float(w[2]), __uint_as_float(w[3])), b0));
+                const float2 y2 = gelu_as2(add2(make_float2(__uint_as_float(w[4]), __uint_as_float(w[5])), b1));
+                const float2 y3 = gelu_as2(add2(make_float2(__uint_as_float(w[6]), __uint_as_float(w[7])), b1));
+                put_tiles(hid + buf * HID_BYTES + (i >> 2) * 16384, row0, 2 * (i & 3), lane, pk2(y0.x, y0.y),
+                          pk2(y1.x, y1.y), pk2(y2.x, y2.y), pk2(y3.x, y3.y));
               }
               put_hid(buf);
             }
@@ -942,12 +988,14 @@ uint8_t* pack_unit(uint8_t* dst, int u, const float* W1, int n1, const float* W2
         for (int kk = 0; kk < 64; ++kk)
           put(dst, n, kk, W2[(size_t)(c * 128 + (i >> 1) * 64 + kk) * TE + (i & 1) * 128 + n]);
   };
-  if (u == 2) {
+  if (u == 2) {                     // the first GEMM two chunks ahead: its accumulator is free before the GELUs are done
     first(0);
-    for (int c = 1; c < 8; ++c) {
+    first(1);
+    for (int c = 2; c < 8; ++c) {
       first(c);
-      second(c - 1);
+      second(c - 2);
     }
+    second(6);
     second(7);
   } else {
     for (int c = 0; c < n_first(u); ++c) first(c);
