@@ -12,9 +12,8 @@
 //     SA:  GEMM xln W_qkv (bf16 out) -> attention (causal) -> GEMM W_o (residual) -> walk_kernel
 //     CA:  GEMM xln W_q -> attention (memory tokens) -> GEMM W_o (residual) -> walk_kernel
 //     FFN: GEMM xln W_1 (GELU, bf16 out) -> GEMM W_2 (residual) -> walk_kernel
-//   GEMM (residual)   the unit's output projection: r and c_b <- bf16(r) for the
-//                     rows that refresh the unit (evo_tc.cuh, EPI_RESID); the walk
-//                     adds r to the residual stream
+//   GEMM (residual)   the unit's output projection: a += r and c_b <- bf16(r) for
+//                     the rows that refresh the unit (evo_tc.cuh, EPI_RESID)
 //   walk_kernel       one warp per row, from the unit just computed to the next
 //                     refreshed cell: the skipped units' cache adds, at step ends
 //                     LN_f, eps = . W_head + b_head, the sampler step (DDPM /
@@ -22,7 +21,8 @@
 //                     LayerNorm of the next refreshed unit -> xln (bf16).  With
 //                     lattices that differ by sample, only the rows that refreshed
 //                     the cell, each to its own lattice's next refreshed cell.
-//                     Caches, r and the stream move with the evict-first policy.
+//                     Caches move with the evict-first policy; the stream is written
+//                     only where it changed.
 // The GEMMs skip 128-row tiles none of whose lattices refresh the unit.  Rows
 // of one lattice are contiguous (samples are ordered by lattice), so with the
 // batch sizes this path serves a 128-row tile rarely mixes lattices.
@@ -73,7 +73,7 @@ bool make_map(CUtensorMap* m, const void* base, long long rows, int K, int box_r
 }
 
 // fp32 matrix [rows][cols], cols contiguous, in boxes of 32 x 32 with the
-// 128-byte swizzle (the residual GEMM's bulk stores of r)
+// 128-byte swizzle (the residual GEMM's bulk reductions into the stream)
 bool make_map_f32(CUtensorMap* m, const void* base, long long rows, int cols) {
   EncodeTiledFn enc = encode_fn();
   if (!enc) return false;
@@ -173,8 +173,7 @@ __global__ void obs_to_bf16_kernel(const float* obs, int ntok, int D, int Dp, __
 struct Walk {
   Lat lat;
   int rows, E, A;
-  float* a;                       // [rows][E] residual stream, fp32
-  const float* r;                 // [rows][E] fp32: output of the unit b0 for the rows that refresh it
+  float* a;                       // [rows][E] residual stream, fp32 (unit b0's output added where its lattice refreshes it)
   __nv_bfloat16* cache;           // [U][rmax][E]
   long long cache_unit;           // elements per unit
   __nv_bfloat16* xln;             // [rows][E]
@@ -196,12 +195,11 @@ struct Walk {
   int* status;                    // device status word (index checks of the debug build)
   // when every sample shares one lattice: per step of the walk, the units that
   // are skipped with a valid cache (host-computed, so the cache loads need not
-  // wait for a lookup), for steps t0 .. t0 + n_umask - 1; and whether b0 refreshes
+  // wait for a lookup), for steps t0 .. t0 + n_umask - 1
   static constexpr int MAX_UMASK = 16;
   uint64_t umask[MAX_UMASK];
   int n_umask;
-  int b0_refresh;                 // -1: look it up per row
-  int t0, b0;                     // the unit whose output the launch adds (b0 < 0: start of the call)
+  int t0, b0;                     // the unit just computed (b0 < 0: start of the call)
   int t1, b1;                     // the next cell some lattice refreshes (t1 = T: none, the call ends)
   // rows of different lattices (walk_kernel<NV, true>): each row is walked
   // only after the cells its own lattice refreshes, straight to its lattice's
@@ -220,19 +218,6 @@ template <int NV>
 __device__ __forceinline__ void ld4(float4 (&v)[NV], const float* src, int lane) {
 #pragma unroll
   for (int j = 0; j < NV; ++j) v[j] = *reinterpret_cast<const float4*>(src + 128 * j + 4 * lane);
-}
-
-// the same with the evict-first (streaming) policy
-template <int NV>
-__device__ __forceinline__ void ld4_cs(float4 (&v)[NV], const float* src, int lane) {
-#pragma unroll
-  for (int j = 0; j < NV; ++j) v[j] = __ldcs(reinterpret_cast<const float4*>(src + 128 * j + 4 * lane));
-}
-
-template <int NV>
-__device__ __forceinline__ void st4_cs(float* dst, int lane, const float4 (&v)[NV]) {
-#pragma unroll
-  for (int j = 0; j < NV; ++j) __stcs(reinterpret_cast<float4*>(dst + 128 * j + 4 * lane), v[j]);
 }
 
 template <int NV>
@@ -262,14 +247,15 @@ __device__ __forceinline__ uint2 pack_bf16x4(float4 v) {
 }
 
 // v += c_k for the units k in [b, bend) that the row's lattice skips at step t
-// and whose cache holds a value, in unit order, up to eight cache rows in flight
+// and whose cache holds a value, in unit order, up to eight cache rows in flight;
+// true if there is one
 template <int NV>
 __device__ __forceinline__ float* trace_row(const Walk& p, int t, int k, int row) {
   return p.trace + (((long long)t * p.lat.U + k) * p.rows + row) * p.E;
 }
 
 template <int NV>
-__device__ __forceinline__ void skip_run(const Walk& p, int sample, int row, int lane, int t, int b, int bend,
+__device__ __forceinline__ bool skip_run(const Walk& p, int sample, int row, int lane, int t, int b, int bend,
                                          float4 (&v)[NV]) {
   const uint64_t range = (bend >= 64 ? ~0ull : (1ull << bend) - 1ull) & ~((1ull << b) - 1ull);
   uint64_t m;                                         // skipped units whose cache holds a value
@@ -294,12 +280,12 @@ __device__ __forceinline__ void skip_run(const Walk& p, int sample, int row, int
       st4<NV>(trace_row<NV>(p, t, k, row), lane, c);
     }
   }
-  // The walk streams the unit caches, r and the residual stream with the
-  // evict-first policy (ld/st .cs): none is read again before hundreds of MB
-  // of other traffic, and the L2 then keeps the GEMM operands (xln, q|k|v,
-  // the hidden layer) that the next kernels read.
+  // The walk streams the unit caches with the evict-first policy (ld .cs): none
+  // is read again before hundreds of MB of other traffic, and the L2 then keeps
+  // the GEMM operands (xln, q|k|v, the hidden layer) that the next kernels read.
   const __nv_bfloat16* base = p.cache + (long long)row * p.E + 4 * lane;
-  if (!dcheck(bend <= p.lat.U && (long long)row * p.E < p.cache_unit, p.status)) return;
+  if (!dcheck(bend <= p.lat.U && (long long)row * p.E < p.cache_unit, p.status)) return false;
+  const bool any = m != 0;
   while (m) {
     constexpr int BATCH = NV >= 4 ? 4 : 8;   // cache rows in flight (registers: BATCH x NV x 8 bytes per lane)
     uint2 raw[BATCH][NV];
@@ -320,6 +306,7 @@ __device__ __forceinline__ void skip_run(const Walk& p, int sample, int row, int
 #pragma unroll
         for (int j = 0; j < NV; ++j) add_bf16x4(v[j], raw[q][j]);
   }
+  return any;
 }
 
 // mean and 1/sqrt(var + eps) of the row (two passes over the registers)
@@ -434,23 +421,24 @@ __device__ __forceinline__ int next_refresh(const Walk& p, int sample, int t, in
 }
 
 // Walk the row from step t, unit b (v = the stream before unit b) to the cell
-// (t1, b1) -- writing the stream and, for that cell's unit, the LayerNorm
-// output -- or, when t1 = T, to the end of the call (x final).
+// (t1, b1) -- writing the stream if it changed (dirty: from the start) and, for
+// that cell's unit, the LayerNorm output -- or, when t1 = T, to the end of the call (x final).
 template <int NV>
 __device__ __forceinline__ void walk_row(const Walk& p, int row, int lane, int t, int b, float4 (&v)[NV], int t1,
-                                         int b1) {
+                                         int b1, bool dirty) {
   const int sample = row / p.lat.H, tok = row - sample * p.lat.H;
   for (;;) {
     const bool last = t == t1;
     const int bend = last ? b1 : p.lat.U;
-    if (b < bend) skip_run<NV>(p, sample, row, lane, t, b, bend, v);
+    if (b < bend) dirty |= skip_run<NV>(p, sample, row, lane, t, b, bend, v);
     if (last) break;
+    dirty = true;
     if (!head_step<NV>(p, row, sample, tok, lane, t, v)) return;   // the call's last step: x is final
     ++t;
     b = 0;
   }
   if (!dcheck(row < p.rows && b1 < p.lat.U && t1 < p.lat.T, p.status)) return;
-  st4_cs<NV>(p.a + (long long)row * p.E, lane, v);
+  if (dirty) st4<NV>(p.a + (long long)row * p.E, lane, v);
   if (lat_refresh(p.lat, sample, b1, t1)) {
     float mean, rstd;
     row_stats<NV>(v, 1.f / (float)p.E, mean, rstd);
@@ -465,9 +453,8 @@ __device__ __forceinline__ void walk_row(const Walk& p, int row, int lane, int t
 // One warp per row: the walk from the launch's position to the next refreshed
 // cell (PER_ROW: the next cell the row's own lattice refreshes).  b0 < 0: the
 // start of a call (x <- noise[0]; a <- x W_in + b_in + P_pos).  Otherwise the
-// rows that refresh unit b0 add its output r (written by the residual GEMM);
-// the walk starts at b0, so rows that skip b0 add its cache (PER_ROW: such
-// rows are already past b0 and do nothing).
+// walk goes on behind unit b0, whose output the residual GEMM has added
+// (PER_ROW: rows that skip b0 are already past it and do nothing).
 template <int NV, bool PER_ROW>
 __global__ void __launch_bounds__(256, 3) walk_kernel(const Walk p) {
   tc::pdl_trigger();
@@ -485,24 +472,12 @@ __global__ void __launch_bounds__(256, 3) walk_kernel(const Walk p) {
     }
     embed<NV>(p, tok, lane, xv, v);
     const int nx = PER_ROW ? next_refresh(p, sample, 0, -1) : p.t1 * 64 + p.b1;
-    walk_row<NV>(p, row, lane, 0, 0, v, nx >> 6, nx & 63);
+    walk_row<NV>(p, row, lane, 0, 0, v, nx >> 6, nx & 63, true);
   } else {
     if (PER_ROW && !lat_refresh(p.lat, sample, p.b0, p.t0)) return;   // the row waits at its own position
-    // the stream, unit b0's output and the lattice bit, loaded together
-    float4 r[NV];
-    ld4_cs<NV>(v, p.a + (long long)row * p.E, lane);
-    ld4_cs<NV>(r, p.r + (long long)row * p.E, lane);
-    if (p.b0_refresh >= 0 ? p.b0_refresh != 0 : lat_refresh(p.lat, sample, p.b0, p.t0)) {
-#pragma unroll
-      for (int j = 0; j < NV; ++j) {
-        v[j].x += r[j].x;
-        v[j].y += r[j].y;
-        v[j].z += r[j].z;
-        v[j].w += r[j].w;
-      }
-    }
+    ld4<NV>(v, p.a + (long long)row * p.E, lane);
     const int nx = PER_ROW ? next_refresh(p, sample, p.t0, p.b0) : p.t1 * 64 + p.b1;
-    walk_row<NV>(p, row, lane, p.t0, p.b0, v, nx >> 6, nx & 63);
+    walk_row<NV>(p, row, lane, p.t0, p.b0, v, nx >> 6, nx & 63, false);
   }
 }
 
@@ -743,7 +718,6 @@ struct WideState {
   __nv_bfloat16* hid = nullptr;     // [rmax][4E]
   __nv_bfloat16* cache = nullptr;   // [U][rmax][E]
   float* a = nullptr;               // [rmax][E]
-  float* rbuf = nullptr;            // [rmax][E]: output of the unit just computed
   __nv_bfloat16* head_wt = nullptr; // [2][A][E] bf16: W_head transposed, then W_in (the row walk's head and embedding)
   float* ln_gb = nullptr;           // [2][U][E]: LayerNorm gain and shift of every unit's branch
   // observation conditioning on the tensor cores: embedding, MLP (Mish), keys|values
@@ -762,7 +736,7 @@ struct WideState {
   CUtensorMap mA_obs, mA_cx, mA_ch, mA_cm;
   // tiled-store maps of the bf16 GEMM outputs (32-row x 64-column boxes)
   CUtensorMap mC_qkv, mC_q, mC_hid, mC_cx, mC_ch, mC_cm;
-  CUtensorMap mC_r;                 // fp32 r (rbuf), 32 x 32 boxes: the residual GEMM's bulk stores
+  CUtensorMap mC_a;                 // fp32 stream, 32 x 32 boxes: the residual GEMM's bulk reductions
   BMaps mB_obs, mB_cw1, mB_cw2, mB_kv;
   // the tile path's keys/values (wide_tile_kv): W_kv^T and bias with the head dims reordered,
   // the timestep tokens' [T][L][2E], the observation tokens' [tokcap][L][2E]
@@ -1015,8 +989,6 @@ int wide_create(WideState** out, const evo_config* c, const float* weights, cons
     return fail(EVO_ERR_OOM);
   if (guarded_malloc(reinterpret_cast<void**>(&w->a), R * E * 4, &w->guards) != cudaSuccess)
     return fail(EVO_ERR_OOM);
-  if (guarded_malloc(reinterpret_cast<void**>(&w->rbuf), R * E * 4, &w->guards) != cudaSuccess)
-    return fail(EVO_ERR_OOM);
   if (cudaMalloc(&w->first, (size_t)max_sched * w->U * sizeof(int)) != cudaSuccess) return fail(EVO_ERR_OOM);
   if (cudaMalloc(&w->mask, (size_t)max_sched * w->T * 2 * sizeof(uint64_t)) != cudaSuccess) return fail(EVO_ERR_OOM);
   // operand rows that no call writes (padding up to a tile) read as zero
@@ -1030,7 +1002,7 @@ int wide_create(WideState** out, const evo_config* c, const float* weights, cons
       !make_map(&w->mB_4e.n128, w->wt_4e, (long long)L * E, 4 * E, 128) ||
       !make_map(&w->mB_4e.n256, w->wt_4e, (long long)L * E, 4 * E, 256) ||
       !make_map(&w->mC_qkv, w->qkv, R, 3 * E, 32) || !make_map(&w->mC_q, w->qkv, R, E, 32) ||
-      !make_map(&w->mC_hid, w->hid, R, 4 * E, 32) || !make_map_f32(&w->mC_r, w->rbuf, R, E))
+      !make_map(&w->mC_hid, w->hid, R, 4 * E, 32) || !make_map_f32(&w->mC_a, w->a, R, E))
     return fail(EVO_ERR_CUDA);
   if (gemm_attr<tc::EPI_BF16, 128>() != cudaSuccess || gemm_attr<tc::EPI_BF16, 256>() != cudaSuccess ||
       gemm_attr<tc::EPI_GELU_BF16, 128>() != cudaSuccess || gemm_attr<tc::EPI_GELU_BF16, 256>() != cudaSuccess ||
@@ -1062,7 +1034,6 @@ void wide_destroy(WideState* w) {
   guarded_free(w->hid);
   guarded_free(w->cache);
   guarded_free(w->a);
-  guarded_free(w->rbuf);
   cudaFree(w->first);
   cudaFree(w->mask);
   cudaFree(w->head_wt);
@@ -1238,7 +1209,6 @@ cudaError_t wide_launch(WideState* w, const WideCall& c, cudaStream_t st) {
   wp.E = E;
   wp.A = w->A;
   wp.a = w->a;
-  wp.r = w->rbuf;
   wp.cache = w->cache;
   wp.cache_unit = w->rmax * E;
   wp.xln = w->xln;
@@ -1291,14 +1261,9 @@ cudaError_t wide_launch(WideState* w, const WideCall& c, cudaStream_t st) {
   wp.per_row = uniform ? 0 : 1;
   auto set_umask = [&]() {
     wp.n_umask = 0;
-    wp.b0_refresh = -1;
     if (!uniform) return;
     wp.n_umask = std::min(Walk::MAX_UMASK, T - wp.t0);
     for (int i = 0; i < wp.n_umask; ++i) wp.umask[i] = skipm[wp.t0 + i];
-    if (wp.b0 >= 0) {
-      const int r = c.S_rows == U ? wp.b0 : wp.b0 / 3;
-      wp.b0_refresh = ((w->force && wp.t0 == 0) || c.S_host[(size_t)r * T + wp.t0]) ? 1 : 0;
-    }
   };
   auto set_next = [&](size_t i) {
     if (i < cells.size()) {
@@ -1325,7 +1290,7 @@ cudaError_t wide_launch(WideState* w, const WideCall& c, cudaStream_t st) {
   g.force = w->force;
   g.status = c.status;
   g.wait_limit = WAIT_POLLS_DEFAULT;
-  g.rout = w->rbuf;
+  g.stream = w->a;
   g.ldr = E;
 
   AttnArgs ap{};
@@ -1371,7 +1336,7 @@ cudaError_t wide_launch(WideState* w, const WideCall& c, cudaStream_t st) {
                      dim3(SA_WARPS * 32), sa_smem, st, ap));
       g.b_row0 = rowE + 3 * E;
       g.bias = wl(w, l, WL_SA_BO);
-      WCK(gemm<tc::EPI_RESID>(w->mA_att, w->mB_e, w->mC_r, g, Rp, E, w->num_sms, pdl, st));
+      WCK(gemm<tc::EPI_RESID>(w->mA_att, w->mB_e, w->mC_a, g, Rp, E, w->num_sms, pdl, st));
       WCK(walk(wp, pdl, st));
     } else if (u == 1) {
       g.K = E;
@@ -1385,7 +1350,7 @@ cudaError_t wide_launch(WideState* w, const WideCall& c, cudaStream_t st) {
                      dim3(SA_WARPS * 32), ca_smem, st, ap));
       g.b_row0 = rowE + 5 * E;
       g.bias = wl(w, l, WL_CA_BO);
-      WCK(gemm<tc::EPI_RESID>(w->mA_att, w->mB_e, w->mC_r, g, Rp, E, w->num_sms, pdl, st));
+      WCK(gemm<tc::EPI_RESID>(w->mA_att, w->mB_e, w->mC_a, g, Rp, E, w->num_sms, pdl, st));
       WCK(walk(wp, pdl, st));
     } else {
       g.K = E;
@@ -1397,7 +1362,7 @@ cudaError_t wide_launch(WideState* w, const WideCall& c, cudaStream_t st) {
       g.K = 4 * E;
       g.b_row0 = l * E;
       g.bias = wl(w, l, WL_FF_B2);
-      WCK(gemm<tc::EPI_RESID>(w->mA_hid, w->mB_4e, w->mC_r, g, Rp, E, w->num_sms, pdl, st));
+      WCK(gemm<tc::EPI_RESID>(w->mA_hid, w->mB_4e, w->mC_a, g, Rp, E, w->num_sms, pdl, st));
       WCK(walk(wp, pdl, st));
     }
   }
