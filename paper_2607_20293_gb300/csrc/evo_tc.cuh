@@ -442,7 +442,7 @@ __global__ void __launch_bounds__(NTHREADS_GEMM, 1) gemm_kernel(const __grid_con
     uint32_t s = 0, ph = 1;                // stage, phase of `empty` that frees it
     for (int tile = blockIdx.x; tile < total; tile += gridDim.x) {
       const int m0 = (tile / n_tiles) * BM, n0 = (tile % n_tiles) * BN;
-      if (!tile_live(g, m0)) continue;
+      if (!__any_sync(0xffffffffu, tile_live(g, m0))) continue;   // (a vote: uniform to the compiler)
       for (int kb = 0; kb < KB; ++kb) {
         mbar_wait(&empty[s], ph, g.status, g.wait_limit);
         if (elect_one()) {
@@ -461,7 +461,7 @@ __global__ void __launch_bounds__(NTHREADS_GEMM, 1) gemm_kernel(const __grid_con
     uint32_t s = 0, ph = 0, it = 0;
     const uint64_t da0 = sw128_desc(su32(smem)), db0 = sw128_desc(su32(smem) + A_BYTES);
     for (int tile = blockIdx.x; tile < total; tile += gridDim.x) {
-      if (!tile_live(g, (tile / n_tiles) * BM)) continue;
+      if (!__any_sync(0xffffffffu, tile_live(g, (tile / n_tiles) * BM))) continue;
       const uint32_t acc = it & 1u;
       mbar_wait(&tempty[acc], ((it >> 1) & 1u) ^ 1u, g.status, g.wait_limit);
       tc_fence_after();

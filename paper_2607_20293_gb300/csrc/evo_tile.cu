@@ -255,6 +255,12 @@ __device__ __forceinline__ void arrive_warp(uint64_t* bar, int lane) {
   if (lane == 0) mbar_arrive1(bar);
 }
 
+// the same value in every lane, and known to the compiler to be
+__device__ __forceinline__ uint64_t uniform64(uint64_t v) {
+  const uint32_t lo = __shfl_sync(0xffffffffu, (uint32_t)v, 0), hi = __shfl_sync(0xffffffffu, (uint32_t)(v >> 32), 0);
+  return ((uint64_t)hi << 32) | lo;
+}
+
 struct Bars {
   uint64_t full[NSLOTS], empty[NSLOTS];   // weight ring
   uint64_t vfull[2], vempty[2];           // vectors of a unit: landed / read (8 warps)
@@ -414,7 +420,7 @@ __global__ void __launch_bounds__(TTHREADS, 1) tile_kernel(const TileParams p) {
         const uint64_t* mk = p.mask + (long long)lattice_of(p, j) * p.T * 2;
         uint64_t nxt = __ldg(mk);
         for (int t = 0; t < p.T; ++t) {
-          uint64_t m = nxt;
+          uint64_t m = uniform64(nxt);
           if (t + 1 < p.T) nxt = __ldg(mk + 2 * (t + 1));
           while (m) {
             const int b = __ffsll((long long)m) - 1, l = b / 3, u = b - 3 * l;
@@ -454,7 +460,7 @@ __global__ void __launch_bounds__(TTHREADS, 1) tile_kernel(const TileParams p) {
         const uint64_t* mk = p.mask + (long long)lattice_of(p, j) * p.T * 2;
         uint64_t nxt = __ldg(mk);
         for (int t = 0; t < p.T; ++t) {
-          uint64_t m = nxt;
+          uint64_t m = uniform64(nxt);
           if (t + 1 < p.T) nxt = __ldg(mk + 2 * (t + 1));
           while (m) {
             const int b = __ffsll((long long)m) - 1, u = b % 3;

@@ -1282,7 +1282,9 @@ cudaError_t wide_launch(WideState* w, const WideCall& c, cudaStream_t st) {
 
   tc::GemmArgs g{};
   g.rows = (int)R;
-  g.S = c.S_dev;
+  // one lattice: every row refreshes every cell of the list, and the GEMMs need no gate (a global load
+  // per tile in each of their roles)
+  g.S = uniform ? nullptr : c.S_dev;
   g.S_stride = one;
   g.T = T;
   g.H = H;
