@@ -982,15 +982,16 @@ bool use_wide(const evo_handle* h, long long samples) {
 }
 
 // The tile path serves calls of more than three rounds of the 4-CTA clusters
-// (36 fit): 112 samples of the 10-action policy at refresh fraction 0.125 / 1.0
-// take 7.6 / 38.9 ms, four cluster rounds 9.4 / 45.6.
+// (36 fit): 108 samples of the 10-action policy at refresh fraction 0.125 / 1.0
+// take 7.1 / 34.5 ms on tiles and 7.1 / 34.1 in three rounds, four rounds 9.4 / 45.6.
 constexpr long long TILE_MIN_SAMPLES = 109;
 bool use_tile(const evo_handle* h, long long samples) { return h->tile && samples >= TILE_MIN_SAMPLES; }
 
 // Where the batch-wide path is the other choice, it stays ahead on one sparse
 // lattice for few samples (a tile adds the skipped units' caches 64 KiB at a
-// time on one SM): 128 / 208 / 256 samples at fraction 0.05 take 3.5 / 4.0 / 4.8
-// ms there and 4.2 / 4.3 / 4.3 on tiles, at 0.125 7.6 / 8.8 / 10.1 and 7.6.
+// time on one SM): 128 / 176 / 208 samples of the 10-action policy at fraction
+// 0.05 take 3.3 / 3.6 / 3.7 ms there and 4.1 on tiles, at 0.08 5.0 / 5.5 / 5.7
+// and 5.5, at 0.125 7.1 / 7.8 / 8.1 and 7.1.
 bool sparse_for_tile(const evo_handle* h, long long samples, int S_rows) {
   if (samples >= 224 || samples * h->H < h->wide_rows) return false;
   const size_t n = (size_t)S_rows * h->T;

@@ -21,8 +21,8 @@
 //                     LayerNorm of the next refreshed unit -> xln (bf16).  With
 //                     lattices that differ by sample, only the rows that refreshed
 //                     the cell, each to its own lattice's next refreshed cell.
-//                     Caches move with the evict-first policy; the stream is written
-//                     only where it changed.
+//                     Caches (and a stream too large for L2) move with the
+//                     evict-first policy; the stream is written only where it changed.
 // The GEMMs skip 128-row tiles none of whose lattices refresh the unit.  Rows
 // of one lattice are contiguous (samples are ordered by lattice), so with the
 // batch sizes this path serves a 128-row tile rarely mixes lattices.
@@ -206,6 +206,7 @@ struct Walk {
   // next refreshed cell (rows that skip (t0, b0) have nothing to do in this
   // launch); one shared lattice: every row to (t1, b1)
   int per_row;
+  int far;                        // the stream is too large to wait in L2: it moves with the evict-first policy
 };
 
 __device__ __forceinline__ float warp_sum(float s) {
@@ -218,6 +219,19 @@ template <int NV>
 __device__ __forceinline__ void ld4(float4 (&v)[NV], const float* src, int lane) {
 #pragma unroll
   for (int j = 0; j < NV; ++j) v[j] = *reinterpret_cast<const float4*>(src + 128 * j + 4 * lane);
+}
+
+// the same with the evict-first (streaming) policy
+template <int NV>
+__device__ __forceinline__ void ld4_cs(float4 (&v)[NV], const float* src, int lane) {
+#pragma unroll
+  for (int j = 0; j < NV; ++j) v[j] = __ldcs(reinterpret_cast<const float4*>(src + 128 * j + 4 * lane));
+}
+
+template <int NV>
+__device__ __forceinline__ void st4_cs(float* dst, int lane, const float4 (&v)[NV]) {
+#pragma unroll
+  for (int j = 0; j < NV; ++j) __stcs(reinterpret_cast<float4*>(dst + 128 * j + 4 * lane), v[j]);
 }
 
 template <int NV>
@@ -438,7 +452,10 @@ __device__ __forceinline__ void walk_row(const Walk& p, int row, int lane, int t
     b = 0;
   }
   if (!dcheck(row < p.rows && b1 < p.lat.U && t1 < p.lat.T, p.status)) return;
-  if (dirty) st4<NV>(p.a + (long long)row * p.E, lane, v);
+  if (dirty) {
+    if (p.far) st4_cs<NV>(p.a + (long long)row * p.E, lane, v);
+    else st4<NV>(p.a + (long long)row * p.E, lane, v);
+  }
   if (lat_refresh(p.lat, sample, b1, t1)) {
     float mean, rstd;
     row_stats<NV>(v, 1.f / (float)p.E, mean, rstd);
@@ -475,7 +492,8 @@ __global__ void __launch_bounds__(256, 3) walk_kernel(const Walk p) {
     walk_row<NV>(p, row, lane, 0, 0, v, nx >> 6, nx & 63, true);
   } else {
     if (PER_ROW && !lat_refresh(p.lat, sample, p.b0, p.t0)) return;   // the row waits at its own position
-    ld4<NV>(v, p.a + (long long)row * p.E, lane);
+    if (p.far) ld4_cs<NV>(v, p.a + (long long)row * p.E, lane);
+    else ld4<NV>(v, p.a + (long long)row * p.E, lane);
     const int nx = PER_ROW ? next_refresh(p, sample, p.t0, p.b0) : p.t1 * 64 + p.b1;
     walk_row<NV>(p, row, lane, p.t0, p.b0, v, nx >> 6, nx & 63, false);
   }
@@ -771,6 +789,11 @@ const float* wl(const WideState* w, int l, int id) {
 }
 
 constexpr long long PDL_MAX_ROWS = 32768;
+// From this size on the stream does not outlive the GEMMs of a unit in L2, and
+// the walk moves it with the evict-first policy, which leaves their operands
+// there.  n_emb 512: 256 samples (16 MiB) 11.70 ms with the policy off, 11.80
+// on; 640 (40 MiB) 24.13 and 24.06; 1,024 (64 MiB) 90.3 and 88.3.
+constexpr long long FAR_STREAM_BYTES = 40ll << 20;
 
 // Launch with programmatic stream serialization: the kernel may begin while
 // its predecessor finishes (every kernel of this path waits for it with
@@ -1259,6 +1282,7 @@ cudaError_t wide_launch(WideState* w, const WideCall& c, cudaStream_t st) {
       }
   }
   wp.per_row = uniform ? 0 : 1;
+  wp.far = R * E * 4 >= FAR_STREAM_BYTES;
   auto set_umask = [&]() {
     wp.n_umask = 0;
     if (!uniform) return;
