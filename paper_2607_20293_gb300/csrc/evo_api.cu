@@ -71,6 +71,7 @@ struct evo_handle {
   long long wide_rows = 1024;
   // tile path (null when the configuration has none or fixes its decomposition)
   TileState* tile = nullptr;
+  int num_sms = 0;
   JobParams tile_base{};              // what evo_get_launch_info reports of it
   int last_path = 0;
   long long last_kernels = 0;
@@ -790,6 +791,7 @@ evo_status evo_create(const float* weights, size_t n_floats, const evo_config* c
       int ts = tile_create(&h->tile, cfg, weights, h->woff, max_batch);
       if (ts == EVO_OK) ts = wide_tile_kv(h->wide, weights, h->kv_time);
       if (ts != EVO_OK) return fail((evo_status)ts);
+      if (cudaDeviceGetAttribute(&h->num_sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return fail(EVO_ERR_CUDA);
       h->tile_base.C = 1;
       h->tile_base.g = 8;
       h->tile_base.sm.total = tile_smem_bytes();
@@ -1000,6 +1002,26 @@ bool sparse_for_tile(const evo_handle* h, long long samples, int S_rows) {
   return 8 * cells < n;
 }
 
+// A population's lattices differ in length, so the choice is by the estimated
+// times of both, longest first on either: a job of c refreshed cells and T steps
+// takes 8 us a step + 4.4 us a cell on a cluster of 4 (a sample each) and 23 +
+// 13.2 on a tile (up to 8 samples), the reference's being the longest.  Push-T
+// shaped, tiles / clusters: 12 candidates x 11 observations of 5 .. 60 % density
+// 33.8 / 22.0 ms, 16 x 16 33.8 / 38.6, 64 x 16 34.1 / 129.6; 119 x 1 of 100 cells
+// 34.1 / 11.4.
+bool population_on_tiles(const evo_handle* h, const uint8_t* S, int P, int N_obs, int S_rows) {
+  const evo_handle::Alt* four = h->n_alt && h->alt[h->n_alt - 1].base.C == 4 ? &h->alt[h->n_alt - 1] : nullptr;
+  if (!four) return true;
+  const size_t n = (size_t)P * S_rows * h->T;
+  const double per = S_rows == h->U ? 1.0 : 3.0, all = (double)h->U * h->T;
+  double cells = all;                                  // of the reference
+  for (size_t i = 0; i < n; ++i) cells += S[i] ? per : 0.0;
+  const double jobs = P + 1.0, tiles = (N_obs + 7) / 8;
+  const double cluster = std::max(8.0 * h->T + 4.4 * all, N_obs * (jobs * 8.0 * h->T + 4.4 * cells) / four->max_clusters);
+  const double tile = std::max(23.0 * h->T + 13.2 * all, tiles * (jobs * 23.0 * h->T + 13.2 * cells) / h->num_sms);
+  return tile < cluster;
+}
+
 // Lattices for a tile-path call.  Calls of wide_rows rows and more are the ones
 // whose device lattices are checked before anything is launched.
 evo_status stage_tile(evo_handle* h, const uint8_t* S, int n_sched, int rows, bool add_ones, long long samples,
@@ -1189,15 +1211,22 @@ evo_status evo_denoise_population(evo_handle* h, const float* obs, const float* 
   if (S_rows != h->U && S_rows != h->L) return EVO_ERR_SCHEDULE;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   const int HA = h->H * h->A;
-  if (use_tile(h, samples)) {
-    const int* err = nullptr;
-    const evo_status s = stage_tile(h, S_pop, P, S_rows, true, samples, st, &err);
-    if (s != EVO_OK) return s;
-    return run_tile(h, obs, noise, h->pop_x, N_obs, P + 1, S_rows, err, st, out_actions, dev_l2);
-  }
-  if (use_wide(h, samples)) {
+  const bool host_checked = use_wide(h, samples);     // such calls' device lattices are checked before any launch
+  if (host_checked) {
     const evo_status s = stage_wide(h, S_pop, P, S_rows, true, st);
     if (s != EVO_OK) return s;
+  }
+  if (use_tile(h, samples)) {
+    const int* err = nullptr;
+    const uint8_t* lat = host_checked ? h->last_sched.data() : (is_device_ptr(S_pop) ? nullptr : S_pop);
+    if (lat && population_on_tiles(h, lat, P, N_obs, S_rows)) {
+      if (!host_checked) {
+        const evo_status s = stage_schedules(h, S_pop, P, S_rows, true, st, &err);
+        if (s != EVO_OK) return s;
+      }
+      return run_tile(h, obs, noise, h->pop_x, N_obs, P + 1, S_rows, err, st, out_actions, dev_l2);
+    }
+  } else if (host_checked) {
     h->last_cond_kernels = 0;                  // the batch-wide sequence computes kv_obs itself
     EVO_CUDA(launch_wide(h, obs, noise, h->pop_x, (int)samples, N_obs, P + 1, S_rows, st));
     EVO_CUDA(launch_pop_dev(h->pop_x, P, N_obs, HA, dev_l2, st));
@@ -1207,8 +1236,10 @@ evo_status evo_denoise_population(evo_handle* h, const float* obs, const float* 
     return finish(h, st);
   }
   const int* err = nullptr;
-  evo_status s = stage_schedules(h, S_pop, P, S_rows, true, st, &err);
-  if (s != EVO_OK) return s;
+  if (!host_checked) {
+    const evo_status s = stage_schedules(h, S_pop, P, S_rows, true, st, &err);
+    if (s != EVO_OK) return s;
+  }
   EVO_CUDA(obs_cond(h, obs, N_obs, h->cond_scratch, h->kv_obs, st));
   Pick pk = pick_decomposition(h, samples);
   JobParams p = *pk.base;

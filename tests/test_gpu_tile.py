@@ -73,16 +73,17 @@ def test_tile_population_edge_lattices(torch, B, empty):
     cfg = synth.config("pusht", n_steps=20, n_layer=2)
     U, T, N = 6, 20, 11
     W = synth.make_weights(cfg, 0)
-    lat = np.zeros((11, U, T), np.uint8)
+    P = 40                            # enough lattices that tiles are the faster choice
+    lat = np.zeros((P, U, T), np.uint8)
     lat[0, 0, 0] = 1                  # the first cell only
     lat[1, U - 1, T - 1] = 1          # the last cell only
     lat[2, :, 0] = 1                  # every unit at step 0, then skips to the end
     lat[3, :, T - 1] = 1
     lat[4] = 1                        # the reference itself; lattice 5: nothing refreshed
-    for p in range(6, 11):
-        lat[p] = synth.bernoulli_schedule(U, T, 0.1 * p, p)
+    for p in range(6, P):
+        lat[p] = synth.bernoulli_schedule(U, T, 0.1 * (p % 11), p)
     obs, noise = synth.make_obs(cfg, N, 81), synth.make_noise(cfg, N, 82)
-    ev = B.Evo(cfg, W, 12 * N, empty=empty)
+    ev = B.Evo(cfg, W, (P + 1) * N, empty=empty)
     x, dev = ev.population(torch.from_numpy(obs).cuda(), torch.from_numpy(noise).cuda(), lat)
     assert on_tiles(ev)
     x, dev = x.cpu().numpy(), dev.cpu().numpy()
@@ -91,8 +92,15 @@ def test_tile_population_edge_lattices(torch, B, empty):
         close(x[p][idx], O.denoise(W, cfg, obs[idx], noise[:, idx], lat[p], policy=empty), f"lattice {p} ({empty})")
     assert dev[4] == 0.0              # the same jobs on the same kernel
     full = x[4]
-    want = np.linalg.norm((x - full[None]).reshape(11, N, -1), axis=2).mean(1)
+    want = np.linalg.norm((x - full[None]).reshape(P, N, -1), axis=2).mean(1)
     assert np.allclose(dev, want, rtol=1e-4, atol=1e-5)
+    # a few short lattices are faster on clusters, whether they come from the host or the device
+    x2, _ = ev.population(torch.from_numpy(obs).cuda(), torch.from_numpy(noise).cuda(), lat[:11])
+    assert not on_tiles(ev) and ev.last_call()["path"] == "cluster"
+    x3, _ = ev.population(torch.from_numpy(obs).cuda(), torch.from_numpy(noise).cuda(), torch.from_numpy(lat[:11]).cuda())
+    assert not on_tiles(ev) and torch.equal(x2, x3)
+    for p in (0, 5, 9):
+        close(x2[p].cpu().numpy()[idx], O.denoise(W, cfg, obs[idx], noise[:, idx], lat[p], policy=empty), f"{p} on clusters")
 
 
 def test_tile_lattice_forms(torch, B):
