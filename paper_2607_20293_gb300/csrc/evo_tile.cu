@@ -449,7 +449,8 @@ __global__ void __launch_bounds__(TTHREADS, 1) tile_kernel(const TileParams p) {
       }
     } else if (warp == 9) {
       // ------------------------------------------------ MMA issue
-      constexpr uint32_t ID = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(TROWS >> 4) << 24) | ((128u >> 3) << 17);
+      constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(TROWS >> 4) << 24);
+      constexpr uint32_t ID128 = IDESC | ((128u >> 3) << 17), ID256 = IDESC | ((256u >> 3) << 17);
       const uint64_t d0 = sw128_desc(0);
       const uint32_t dhi = (uint32_t)(d0 >> 32), dlo = (uint32_t)d0;     // + (address >> 4)
       const uint32_t dx = dlo + (su32(xln) >> 4), dh = dlo + (su32(hid) >> 4), dr = dlo + (su32(ring) >> 4);
@@ -473,47 +474,64 @@ __global__ void __launch_bounds__(TTHREADS, 1) tile_kernel(const TileParams p) {
 #pragma unroll 1
             for (int i = 0; i < n_ops; ++i) {
               const bool first = u == 2 ? i < 3 || ((i & 1) == 0 && i < 14) : i < nf;
-              uint32_t da, d, sa, sd, acc, bdone;       // A, D and their steps per slot
               if (first) {
                 const uint32_t a = na & 1u;
                 wait(bae + 8 * a, ((na >> 1) & 1u) ^ 1u);
-                da = dx;
-                sa = 0;                                 // K block: the slot
-                d = tA + a * 128;
-                sd = 0;
-                acc = 0;
-                bdone = baf + 8 * a;
+                tc_fence_after();
                 ++na;
+#pragma unroll 1
+                for (uint32_t k = 0; k < 4; ++k) {      // K block k
+                  wait(bfull + 8 * s, ph);
+                  tc_fence_after();
+                  const uint32_t ak = dx + k * (16384 >> 4), bk = dr + s * (SLOT >> 4);
+                  if (elect_one()) {
+#pragma unroll
+                    for (uint32_t e = 0; e < 4; ++e)
+                      mma_f16(tA + a * 128, desc64(ak + 2 * e, dhi), desc64(bk + 2 * e, dhi), ID128, k | e);
+                    commit(bempty + 8 * s);
+                    if (k == 3) commit(baf + 8 * a);
+                  }
+                  next_slot();
+                }
               } else {
                 const uint32_t buf = c2 & 1u;
                 wait(bhr + 8 * buf, nh & 1u);
-                da = dh + buf * (HID_BYTES >> 4);
-                sa = 1;                                 // K block: the slot / 2, columns 128 (slot & 1)
-                d = tR;
-                sd = 128;
-                acc = c2 > 0;
-                bdone = bhe + 8 * buf;
-                nh += buf;                              // the buffers alternate
-                ++c2;
-              }
-              tc_fence_after();
-#pragma unroll 1
-              for (uint32_t k = 0; k < 4; ++k) {
-                wait(bfull + 8 * s, ph);
                 tc_fence_after();
-                const uint32_t kb = k >> sa, ak = da + kb * (16384 >> 4), bk = dr + s * (SLOT >> 4);
-                const uint32_t dk = d + (k & 1u) * sd;
-                if (elect_one()) {
+#pragma unroll 1
+                for (uint32_t k = 0; k < 2; ++k) {      // K block k: its 256 columns in two slots
+                  const uint32_t s0 = s, p0 = ph;
+                  next_slot();
+                  const uint32_t s1 = s, p1 = ph;
+                  next_slot();
+                  wait(bfull + 8 * s0, p0);
+                  wait(bfull + 8 * s1, p1);
+                  tc_fence_after();
+                  const uint32_t ak = dh + buf * (HID_BYTES >> 4) + k * (16384 >> 4);
+                  const uint32_t b0 = dr + s0 * (SLOT >> 4), b1 = dr + s1 * (SLOT >> 4), acc = (uint32_t)c2 | k;
+                  if (elect_one()) {
+                    // one MMA of 256 columns takes 128 cycles, two of 128 take
+                    // 196; a pair that wraps around the ring has to
+                    if (s1) {
 #pragma unroll
-                  for (uint32_t e = 0; e < 4; ++e)
-                    mma_f16(dk, desc64(ak + 2 * e, dhi), desc64(bk + 2 * e, dhi), ID, acc | kb | e);
-                  commit(bempty + 8 * s);
-                  if (k == 3) {
-                    commit(bdone);
-                    if (i == n_ops - 1) commit(brf);
+                      for (uint32_t e = 0; e < 4; ++e)
+                        mma_f16(tR, desc64(ak + 2 * e, dhi), desc64(b0 + 2 * e, dhi), ID256, acc | e);
+                    } else {
+#pragma unroll
+                      for (uint32_t e = 0; e < 4; ++e) {
+                        mma_f16(tR, desc64(ak + 2 * e, dhi), desc64(b0 + 2 * e, dhi), ID128, acc | e);
+                        mma_f16(tR + 128, desc64(ak + 2 * e, dhi), desc64(b1 + 2 * e, dhi), ID128, acc | e);
+                      }
+                    }
+                    commit(bempty + 8 * s0);
+                    commit(bempty + 8 * s1);
+                    if (k == 1) {
+                      commit(bhe + 8 * buf);
+                      if (i == n_ops - 1) commit(brf);
+                    }
                   }
                 }
-                next_slot();
+                nh += buf;                              // the buffers alternate
+                ++c2;
               }
             }
             ++units;
