@@ -620,7 +620,8 @@ def run_population(args, pool, workers):
         "roofline": {"bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
                      "traffic": recorded_traffic("population"), "peak_source": peak_src,
                      "kernel": ("batch-wide launch sequence of one call (tcgen05 GEMMs, attention, row kernels)"
-                                if path == "wide" else "evo::job_kernel (persistent cluster loop)"),
+                                if path == "wide" else "evo::tile_kernel (a block per 8 samples of a lattice)"
+                                if info["cluster"] == 1 else "evo::job_kernel (persistent cluster loop)"),
                      "algorithmic_per_launch": flops, "kernel_ms": kern_ms},
         "e2e": {"value": P * N * 1000.0 / statistics.mean(e2e), "unit": "chunks/s",
                 "h2d_bytes_per_step": int(obs.nbytes + noise.nbytes), "d2h_bytes_per_step": int(h_dev.numel() * 4)},
