@@ -24,7 +24,8 @@
 //     warp refresh the unit) and stores the unit's bf16 cache (Eq. 1) for the
 //     rows that refresh the unit.
 // With two accumulators the epilogue of one tile overlaps the main loop of the
-// next.  BN = 256 for large problems, 128 when that leaves SMs idle.
+// next.  BN = 256 for large problems, 128 when that leaves SMs idle, 64 (residual
+// mode) while even those tiles fit the chip at once.
 //
 // Every wait on an mbarrier is bounded: on expiry the thread records
 // ST_TIMEOUT in the status word and carries on, so the kernel always ends.
@@ -53,7 +54,7 @@ template <int BN>
 struct TileCfg {
   static constexpr int B_BYTES = BN * BK * 2;
   static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
-  static constexpr int STAGES = BN == 256 ? 4 : 6;
+  static constexpr int STAGES = BN == 256 ? 4 : (BN == 128 ? 6 : 8);
   // alignment slack, stages, epilogue staging, barriers
   static constexpr int SMEM_BYTES = 1024 + STAGES * STAGE_BYTES + EPI_STG_BYTES + 256;
   static constexpr int TMEM_COLS = 2 * BN;                                // two accumulators

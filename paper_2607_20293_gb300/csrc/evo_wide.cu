@@ -717,9 +717,9 @@ cudaError_t attn_attr() {
 }  // namespace
 
 // ---------------------------------------------------------------- state
-// B operands: one tensor map per weight matrix and tile width
+// B operands: one tensor map per weight matrix and tile width (64: the residual mode's alone)
 struct BMaps {
-  CUtensorMap n128, n256;
+  CUtensorMap n64, n128, n256;
 };
 
 struct WideState {
@@ -823,7 +823,19 @@ cudaError_t gemm(const CUtensorMap& ma, const BMaps& mb, const CUtensorMap& mc, 
     const int total = m_tiles * (N / 256);
     return launch_pdl(pdl, tc::gemm_kernel<MODE, 256>, dim3(std::min(total, num_sms)), dim3(tc::NTHREADS_GEMM),
                       tc::TileCfg<256>::SMEM_BYTES, st, ma, mb.n256, mc, g, m_tiles, N / 256);
-  } else {
+  }
+  if constexpr (MODE == tc::EPI_RESID) {
+    // few tiles: a 64-column one takes in less (24 KiB a stage for 32) and its
+    // epilogue is half as long.  n_emb 512, 10 steps at full refresh: 32 samples
+    // 8.51 -> 7.80 ms, 50 9.32 -> 8.74, 75 9.65 -> 9.09.  (The bias mode stores
+    // 64-column blocks, so half of its epilogue warps would idle: 8.90 at 50.)
+    if (m_tiles * (N / 64) <= num_sms) {
+      const int total = m_tiles * (N / 64);
+      return launch_pdl(pdl, tc::gemm_kernel<MODE, 64>, dim3(total), dim3(tc::NTHREADS_GEMM),
+                        tc::TileCfg<64>::SMEM_BYTES, st, ma, mb.n64, mc, g, m_tiles, N / 64);
+    }
+  }
+  {
     const int total = m_tiles * (N / 128);
     return launch_pdl(pdl, tc::gemm_kernel<MODE, 128>, dim3(std::min(total, num_sms)), dim3(tc::NTHREADS_GEMM),
                       tc::TileCfg<128>::SMEM_BYTES, st, ma, mb.n128, mc, g, m_tiles, N / 128);
@@ -1020,6 +1032,8 @@ int wide_create(WideState** out, const evo_config* c, const float* weights, cons
   cudaMemset(w->hid, 0, R * 4 * E * 2);
   if (!make_map(&w->mA_xln, w->xln, R, E, tc::BM) || !make_map(&w->mA_att, w->att, R, E, tc::BM) ||
       !make_map(&w->mA_hid, w->hid, R, 4 * E, tc::BM) ||
+      !make_map(&w->mB_e.n64, w->wt_e, (long long)L * 10 * E, E, 64) ||
+      !make_map(&w->mB_4e.n64, w->wt_4e, (long long)L * E, 4 * E, 64) ||
       !make_map(&w->mB_e.n128, w->wt_e, (long long)L * 10 * E, E, 128) ||
       !make_map(&w->mB_e.n256, w->wt_e, (long long)L * 10 * E, E, 256) ||
       !make_map(&w->mB_4e.n128, w->wt_4e, (long long)L * E, 4 * E, 128) ||
@@ -1029,7 +1043,7 @@ int wide_create(WideState** out, const evo_config* c, const float* weights, cons
     return fail(EVO_ERR_CUDA);
   if (gemm_attr<tc::EPI_BF16, 128>() != cudaSuccess || gemm_attr<tc::EPI_BF16, 256>() != cudaSuccess ||
       gemm_attr<tc::EPI_GELU_BF16, 128>() != cudaSuccess || gemm_attr<tc::EPI_GELU_BF16, 256>() != cudaSuccess ||
-      gemm_attr<tc::EPI_RESID, 128>() != cudaSuccess || gemm_attr<tc::EPI_RESID, 256>() != cudaSuccess ||
+      gemm_attr<tc::EPI_RESID, 64>() != cudaSuccess || gemm_attr<tc::EPI_RESID, 128>() != cudaSuccess || gemm_attr<tc::EPI_RESID, 256>() != cudaSuccess ||
       gemm_attr<tc::EPI_MISH_BF16, 128>() != cudaSuccess || gemm_attr<tc::EPI_MISH_BF16, 256>() != cudaSuccess ||
       gemm_attr<tc::EPI_F32, 128>() != cudaSuccess || gemm_attr<tc::EPI_F32, 256>() != cudaSuccess)
     return fail(EVO_ERR_CUDA);

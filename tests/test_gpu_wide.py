@@ -193,3 +193,23 @@ def test_repeated_calls_replay_the_captured_sequence(torch, B):
         got3 = ev.denoise(d_obs, d_noise, S2, out=out).cpu().numpy()
     check(got3, O.denoise(W, cfg, obs3, noise, S2), "new inputs in the same buffers")
     assert ev.status() == B.OK
+
+
+# n_emb 512: 64-column output-projection tiles while they fit the chip at once
+# (19 row tiles of 128: up to 76 samples of 32 rows), 128 beyond
+@pytest.mark.parametrize("n", [1, 76, 77])
+def test_wide_small_tiles_of_the_output_projections(torch, B, n):
+    cfg = synth.config("scale1024", n_steps=10, n_layer=2)
+    W = synth.make_weights(cfg, 0)
+    obs, noise = synth.make_obs(cfg, n, 61), synth.make_noise(cfg, n, 62)
+    S = synth.bernoulli_schedule(6, 10, 0.6, 63)
+    ev = B.Evo(cfg, W, n, wide_rows=1)
+    got = ev.denoise(torch.from_numpy(obs).cuda(), torch.from_numpy(noise).cuda(), S).cpu().numpy()
+    assert ev.last_call()["path"] == "wide"
+    idx = sorted({0, n // 2, n - 1})
+    want = O.denoise(W, cfg, obs[idx], noise[:, idx], S)
+    # 2-norm over all actions: bf16 operands round by 2^-9 per product, and six units
+    # of two layers add up to a few times that; single actions of a 10-step loop are
+    # off by more (x0 = (x - s eps) / sqrt(abar), a factor 7 at the first step, then
+    # few steps to correct it: 0.031 at n = 77 on the 128-column tiles)
+    assert np.linalg.norm(got[idx] - want) <= 1e-2 * np.linalg.norm(want)
