@@ -1037,7 +1037,7 @@ evo_status stage_tile(evo_handle* h, const uint8_t* S, int n_sched, int rows, bo
 evo_status run_tile(evo_handle* h, const float* obs, const float* noise, float* out, int N, int n_sched, int S_rows,
                     const int* err, cudaStream_t st, float* actions = nullptr, float* dev = nullptr) {
   long long n = 0;
-  EVO_CUDA(wide_condition(h->wide, obs, N, nullptr, true, h->status, st, &n));
+  EVO_CUDA(wide_condition(h->wide, obs, N, nullptr, true, h->status, true, st, &n));
   TileCall c{};
   EVO_CUDA(wide_masks(h->wide, h->sched, S_rows, n_sched, st, &c.mask));
   n += 2 + (err ? 1 : 0);

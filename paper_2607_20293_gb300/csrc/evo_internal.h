@@ -304,8 +304,8 @@ cudaError_t wide_run(WideState* w, const WideCall& c);
 // tokens' keys/values (to kv_obs unless null; tile: to the tile path's bf16
 // copy; *launches += the kernels launched) and the lattices'
 // per-step bitmasks [n_sched][T][2] (units refreshed, units whose cache holds a value)
-cudaError_t wide_condition(WideState* w, const float* obs, int n, float* kv_obs, bool tile, int* status, cudaStream_t st,
-                           long long* launches);
+cudaError_t wide_condition(WideState* w, const float* obs, int n, float* kv_obs, bool tile, int* status, bool pdl,
+                           cudaStream_t st, long long* launches);
 cudaError_t wide_masks(WideState* w, const uint8_t* S_dev, int S_rows, int n_sched, cudaStream_t st,
                        const uint64_t** mask);
 // the tile path's keys/values: weights and buffers, the timestep tokens' copy (from kv_time, fp32 on the device)

@@ -786,6 +786,7 @@ const float* wl(const WideState* w, int l, int id) {
   return w->wf32 + w->woff[W_LAYER0] + (long long)l * w->woff[W_LAYER_STRIDE] + w->woff[id];
 }
 
+constexpr long long GRAPH_PDL_MAX_ROWS = 32768;
 // From this size on the stream does not outlive the GEMMs of a unit in L2, and
 // the walk moves it with the evict-first policy, which leaves their operands
 // there.  n_emb 512: 256 samples (16 MiB) 11.70 ms with the policy off, 11.80
@@ -798,10 +799,9 @@ constexpr long long FAR_STREAM_BYTES = 40ll << 20;
 // The row walk and the attention kernels trigger it only by ending: a GEMM that
 // starts while they still have blocks to place takes whole SMs to wait on.
 // n_emb 512, 10 steps at full refresh, against a trigger at their start: 50 samples
-// 8.78 -> 8.70 ms, 256 15.71 -> 15.40, 500 24.63 -> 24.33.  Without the
-// attribute 50 take 10.6, 256 18.3, 1,024 48.3 against 45.5.
+// 8.78 -> 8.70 ms, 256 15.71 -> 15.40, 500 24.63 -> 24.33.
 template <typename... KArgs, typename... Args>
-cudaError_t launch_pdl(void (*k)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+cudaError_t launch_pdl(bool pdl, void (*k)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
                        Args... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
@@ -810,7 +810,7 @@ cudaError_t launch_pdl(void (*k)(KArgs...), dim3 grid, dim3 block, size_t smem, 
   cfg.stream = st;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
+  at[0].val.programmaticStreamSerializationAllowed = pdl ? 1 : 0;
   cfg.attrs = at;
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, k, args...);
@@ -819,11 +819,11 @@ cudaError_t launch_pdl(void (*k)(KArgs...), dim3 grid, dim3 block, size_t smem, 
 // mc: the output's tiled-store map (bf16 modes; the other modes ignore it)
 template <int MODE>
 cudaError_t gemm(const CUtensorMap& ma, const BMaps& mb, const CUtensorMap& mc, const tc::GemmArgs& g, int rows_p,
-                 int N, int num_sms, cudaStream_t st) {
+                 int N, int num_sms, bool pdl, cudaStream_t st) {
   const int m_tiles = rows_p / tc::BM;
   if (N % 256 == 0 && m_tiles * (N / 256) >= num_sms) {
     const int total = m_tiles * (N / 256);
-    return launch_pdl(tc::gemm_kernel<MODE, 256>, dim3(std::min(total, num_sms)), dim3(tc::NTHREADS_GEMM),
+    return launch_pdl(pdl, tc::gemm_kernel<MODE, 256>, dim3(std::min(total, num_sms)), dim3(tc::NTHREADS_GEMM),
                       tc::TileCfg<256>::SMEM_BYTES, st, ma, mb.n256, mc, g, m_tiles, N / 256);
   }
   if constexpr (MODE == tc::EPI_RESID) {
@@ -833,13 +833,13 @@ cudaError_t gemm(const CUtensorMap& ma, const BMaps& mb, const CUtensorMap& mc, 
     // 64-column blocks, so half of its epilogue warps would idle: 8.90 at 50.)
     if (m_tiles * (N / 64) <= num_sms) {
       const int total = m_tiles * (N / 64);
-      return launch_pdl(tc::gemm_kernel<MODE, 64>, dim3(total), dim3(tc::NTHREADS_GEMM),
+      return launch_pdl(pdl, tc::gemm_kernel<MODE, 64>, dim3(total), dim3(tc::NTHREADS_GEMM),
                         tc::TileCfg<64>::SMEM_BYTES, st, ma, mb.n64, mc, g, m_tiles, N / 64);
     }
   }
   {
     const int total = m_tiles * (N / 128);
-    return launch_pdl(tc::gemm_kernel<MODE, 128>, dim3(std::min(total, num_sms)), dim3(tc::NTHREADS_GEMM),
+    return launch_pdl(pdl, tc::gemm_kernel<MODE, 128>, dim3(std::min(total, num_sms)), dim3(tc::NTHREADS_GEMM),
                       tc::TileCfg<128>::SMEM_BYTES, st, ma, mb.n128, mc, g, m_tiles, N / 128);
   }
 }
@@ -850,14 +850,14 @@ cudaError_t gemm_attr() {
                               tc::TileCfg<BN>::SMEM_BYTES);
 }
 
-cudaError_t walk(const Walk& p, cudaStream_t st) {
+cudaError_t walk(const Walk& p, bool pdl, cudaStream_t st) {
   const dim3 grid((p.rows + 7) / 8), block(256);
   if (p.E == 256)
-    return p.per_row ? launch_pdl(walk_kernel<2, true>, grid, block, 0, st, p)
-                     : launch_pdl(walk_kernel<2, false>, grid, block, 0, st, p);
+    return p.per_row ? launch_pdl(pdl, walk_kernel<2, true>, grid, block, 0, st, p)
+                     : launch_pdl(pdl, walk_kernel<2, false>, grid, block, 0, st, p);
   if (p.E == 512)
-    return p.per_row ? launch_pdl(walk_kernel<4, true>, grid, block, 0, st, p)
-                     : launch_pdl(walk_kernel<4, false>, grid, block, 0, st, p);
+    return p.per_row ? launch_pdl(pdl, walk_kernel<4, true>, grid, block, 0, st, p)
+                     : launch_pdl(pdl, walk_kernel<4, false>, grid, block, 0, st, p);
   return cudaErrorInvalidValue;
 }
 
@@ -1097,8 +1097,8 @@ const GuardList* wide_guards(const WideState* w) { return &w->guards; }
 long long wide_last_launches(const WideState* w) { return w ? w->launches : 0; }
 
 // Observation tokens of n samples -> keys/values: a chain of five or six kernels.
-cudaError_t wide_condition(WideState* w, const float* obs, int n, float* kv_obs, bool tile, int* status, cudaStream_t st,
-                           long long* launches) {
+cudaError_t wide_condition(WideState* w, const float* obs, int n, float* kv_obs, bool tile, int* status, bool pdl,
+                           cudaStream_t st, long long* launches) {
   const int E = w->E, L = w->L;
   cudaError_t e;
 #define WCK(x)                    \
@@ -1113,7 +1113,7 @@ cudaError_t wide_condition(WideState* w, const float* obs, int n, float* kv_obs,
   const int ntok = n * w->n_obs;
   const int tp = (ntok + tc::BM - 1) / tc::BM * tc::BM;
   const long long nel = (long long)ntok * w->Dp;
-  WCK(launch_pdl(obs_to_bf16_kernel, dim3((unsigned)std::min<long long>((nel + 255) / 256, 4096)), dim3(256), 0,
+  WCK(launch_pdl(pdl, obs_to_bf16_kernel, dim3((unsigned)std::min<long long>((nel + 255) / 256, 4096)), dim3(256), 0,
                  st, obs, ntok, w->D, w->Dp, w->obs16));
   tc::GemmArgs q{};
   q.rows = ntok;
@@ -1125,29 +1125,29 @@ cudaError_t wide_condition(WideState* w, const float* obs, int n, float* kv_obs,
   q.rbias_mod = w->n_obs;
   q.out = w->cx16;
   q.ldo = E;
-  WCK(gemm<tc::EPI_BF16>(w->mA_obs, w->mB_obs, w->mC_cx, q, tp, E, w->num_sms, st));
+  WCK(gemm<tc::EPI_BF16>(w->mA_obs, w->mB_obs, w->mC_cx, q, tp, E, w->num_sms, pdl, st));
   q.rbias = nullptr;
   q.K = E;
   q.bias = w->wf32 + w->woff[W_CM_B1];
   q.out = w->ch16;
   q.ldo = 4 * E;
-  WCK(gemm<tc::EPI_MISH_BF16>(w->mA_cx, w->mB_cw1, w->mC_ch, q, tp, 4 * E, w->num_sms, st));
+  WCK(gemm<tc::EPI_MISH_BF16>(w->mA_cx, w->mB_cw1, w->mC_ch, q, tp, 4 * E, w->num_sms, pdl, st));
   q.K = 4 * E;
   q.bias = w->wf32 + w->woff[W_CM_B2];
   q.out = w->cm16;
   q.ldo = E;
-  WCK(gemm<tc::EPI_BF16>(w->mA_ch, w->mB_cw2, w->mC_cm, q, tp, E, w->num_sms, st));
+  WCK(gemm<tc::EPI_BF16>(w->mA_ch, w->mB_cw2, w->mC_cm, q, tp, E, w->num_sms, pdl, st));
   q.K = E;
   q.ldo = L * 2 * E;
   if (kv_obs) {
     q.bias = w->bkv;
     q.out32 = kv_obs;
-    WCK(gemm<tc::EPI_F32>(w->mA_cm, w->mB_kv, w->mC_cm, q, tp, L * 2 * E, w->num_sms, st));
+    WCK(gemm<tc::EPI_F32>(w->mA_cm, w->mB_kv, w->mC_cm, q, tp, L * 2 * E, w->num_sms, pdl, st));
   }
   if (tile) {
     q.bias = w->tkv_b;
     q.out = w->tkv_obs;
-    WCK(gemm<tc::EPI_BF16>(w->mA_cm, w->mB_tkv, w->mC_tkv, q, tp, L * 2 * E, w->num_sms, st));
+    WCK(gemm<tc::EPI_BF16>(w->mA_cm, w->mB_tkv, w->mC_tkv, q, tp, L * 2 * E, w->num_sms, pdl, st));
   }
 #undef WCK
   return cudaSuccess;
@@ -1164,7 +1164,7 @@ cudaError_t wide_masks(WideState* w, const uint8_t* S_dev, int S_rows, int n_sch
   lat.T = w->T;
   lat.force = w->force;
   *mask = w->mask;
-  return launch_pdl(first_kernel, dim3(n_sched), dim3(64), 0, st, lat, n_sched, w->first, w->mask);
+  return launch_pdl(false, first_kernel, dim3(n_sched), dim3(64), 0, st, lat, n_sched, w->first, w->mask);
 }
 
 int wide_tile_kv(WideState* w, const float* weights, const float* kv_time) {
@@ -1206,6 +1206,12 @@ cudaError_t wide_launch(WideState* w, const WideCall& c, cudaStream_t st) {
   const int E = w->E, L = w->L, U = w->U, T = w->T, H = w->H;
   const long long R = (long long)c.samples * H;
   const int Rp = (int)((R + tc::BM - 1) / tc::BM * tc::BM);
+  // Programmatic dependent launch hides the gap between kernels: 10 steps at full
+  // refresh, n_emb 512, 50 samples 10.6 -> 8.7 ms, 1,024 48.3 -> 45.5 (100 steps
+  // at 0.125 88.1 -> 86.7).  In a replayed graph the gaps of the largest batches
+  // are hidden without it: 1,024 at 0.125 83.8 ms, and 86.1 with it.
+  const bool captured = w->cap_stream && st == w->cap_stream;
+  const bool pdl = !captured || R < GRAPH_PDL_MAX_ROWS;
   long long n = 0;
   cudaError_t e;
 #define WCK(x)                    \
@@ -1236,8 +1242,8 @@ cudaError_t wide_launch(WideState* w, const WideCall& c, cudaStream_t st) {
   lat.H = H;
   lat.per_sched = c.per_sched;
   lat.force = w->force;
-  if (c.obs && (e = wide_condition(w, c.obs, c.obs_mod, c.kv_obs, false, c.status, st, &n)) != cudaSuccess) return e;
-  WCK(launch_pdl(first_kernel, dim3(c.n_sched), dim3(64), 0, st, lat, c.n_sched, w->first, w->mask));
+  if (c.obs && (e = wide_condition(w, c.obs, c.obs_mod, c.kv_obs, false, c.status, pdl, st, &n)) != cudaSuccess) return e;
+  WCK(launch_pdl(pdl, first_kernel, dim3(c.n_sched), dim3(64), 0, st, lat, c.n_sched, w->first, w->mask));
 
   Walk wp{};
   wp.lat = lat;
@@ -1315,7 +1321,7 @@ cudaError_t wide_launch(WideState* w, const WideCall& c, cudaStream_t st) {
   wp.b0 = -1;
   set_next(0);
   set_umask();
-  WCK(walk(wp, st));
+  WCK(walk(wp, pdl, st));
 
   tc::GemmArgs g{};
   g.rows = (int)R;
@@ -1369,40 +1375,40 @@ cudaError_t wide_launch(WideState* w, const WideCall& c, cudaStream_t st) {
       g.bias = wl(w, l, WL_SA_BQKV);
       g.out = w->qkv;
       g.ldo = 3 * E;
-      WCK(gemm<tc::EPI_BF16>(w->mA_xln, w->mB_e, w->mC_qkv, g, Rp, 3 * E, w->num_sms, st));
+      WCK(gemm<tc::EPI_BF16>(w->mA_xln, w->mB_e, w->mC_qkv, g, Rp, 3 * E, w->num_sms, pdl, st));
       ap.qkv = w->qkv;
-      WCK(launch_pdl(H == 32 ? attn_mma_kernel<2, false> : attn_mma_kernel<1, false>, attn_grid,
+      WCK(launch_pdl(pdl, H == 32 ? attn_mma_kernel<2, false> : attn_mma_kernel<1, false>, attn_grid,
                      dim3(SA_WARPS * 32), sa_smem, st, ap));
       g.b_row0 = rowE + 3 * E;
       g.bias = wl(w, l, WL_SA_BO);
-      WCK(gemm<tc::EPI_RESID>(w->mA_att, w->mB_e, w->mC_a, g, Rp, E, w->num_sms, st));
-      WCK(walk(wp, st));
+      WCK(gemm<tc::EPI_RESID>(w->mA_att, w->mB_e, w->mC_a, g, Rp, E, w->num_sms, pdl, st));
+      WCK(walk(wp, pdl, st));
     } else if (u == 1) {
       g.K = E;
       g.b_row0 = rowE + 4 * E;
       g.bias = wl(w, l, WL_CA_BQ);
       g.out = w->qkv;
       g.ldo = E;
-      WCK(gemm<tc::EPI_BF16>(w->mA_xln, w->mB_e, w->mC_q, g, Rp, E, w->num_sms, st));
+      WCK(gemm<tc::EPI_BF16>(w->mA_xln, w->mB_e, w->mC_q, g, Rp, E, w->num_sms, pdl, st));
       ap.qkv = w->qkv;
-      WCK(launch_pdl(H == 32 ? attn_mma_kernel<2, true> : attn_mma_kernel<1, true>, attn_grid,
+      WCK(launch_pdl(pdl, H == 32 ? attn_mma_kernel<2, true> : attn_mma_kernel<1, true>, attn_grid,
                      dim3(SA_WARPS * 32), ca_smem, st, ap));
       g.b_row0 = rowE + 5 * E;
       g.bias = wl(w, l, WL_CA_BO);
-      WCK(gemm<tc::EPI_RESID>(w->mA_att, w->mB_e, w->mC_a, g, Rp, E, w->num_sms, st));
-      WCK(walk(wp, st));
+      WCK(gemm<tc::EPI_RESID>(w->mA_att, w->mB_e, w->mC_a, g, Rp, E, w->num_sms, pdl, st));
+      WCK(walk(wp, pdl, st));
     } else {
       g.K = E;
       g.b_row0 = rowE + 6 * E;
       g.bias = wl(w, l, WL_FF_B1);
       g.out = w->hid;
       g.ldo = 4 * E;
-      WCK(gemm<tc::EPI_GELU_BF16>(w->mA_xln, w->mB_e, w->mC_hid, g, Rp, 4 * E, w->num_sms, st));
+      WCK(gemm<tc::EPI_GELU_BF16>(w->mA_xln, w->mB_e, w->mC_hid, g, Rp, 4 * E, w->num_sms, pdl, st));
       g.K = 4 * E;
       g.b_row0 = l * E;
       g.bias = wl(w, l, WL_FF_B2);
-      WCK(gemm<tc::EPI_RESID>(w->mA_hid, w->mB_4e, w->mC_a, g, Rp, E, w->num_sms, st));
-      WCK(walk(wp, st));
+      WCK(gemm<tc::EPI_RESID>(w->mA_hid, w->mB_4e, w->mC_a, g, Rp, E, w->num_sms, pdl, st));
+      WCK(walk(wp, pdl, st));
     }
   }
 #undef WCK
