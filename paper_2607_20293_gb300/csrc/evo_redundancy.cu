@@ -12,11 +12,9 @@
 //   w1     : mean |sort(a_t) - sort(a_t')|          (Wasserstein-1 of the entries)
 // and d_{r,b,t} = 1/(T-1) sum_{t' != t} of the term; d_{b,t} = mean over r.
 //
-// Pair kernels: the T rows of a (b, r) are streamed through shared memory in
+// Pair kernel: a block per (b, r) streams its T rows through shared memory in
 // chunks; every thread owns a register tile of (t, t') pairs of the symmetric
-// matrix.  ordered_pair_kernel (a block per (b, r)) keeps every sum in index
-// order; sorted_pair_kernel (Wasserstein-1, a cluster of 1..8 blocks per (b, r))
-// cuts the entries over blocks and threads.  Per-sample maps go to scratch and
+// matrix and keeps every sum in entry order.  Per-sample maps go to scratch and
 // are averaged in a second pass in a fixed order (deterministic).
 //
 // Guided sampling: one block per schedule.  The Eq. 7 weights are taken in
@@ -36,191 +34,17 @@ namespace evo {
 
 namespace {
 
-constexpr int RM_THREADS = 192;
 constexpr int RM_MAX_T = 128;
-constexpr int RM_STAGES = 3;
 
 enum { M_COS = 0, M_MSE = 1, M_L1 = 2, M_W1 = 3 };
-
-// Entries per chunk: 64, and 256 for T <= 32, whose few tiles leave the threads
-// to more groups of 16-byte columns.
-inline int pair_chunk(int T) { return T > 32 ? 64 : 256; }
-// eight rows of a chunk and 16 bytes of padding: a thread addresses its eight
-// rows with immediates, and neighbouring groups of rows start in distinct banks
-__host__ __device__ constexpr int pair_group(int ch) { return 8 * ch + 4; }
-
-// the chunk ring; the threads' tiles (64 sums each) take its place after the last chunk
-size_t pair_smem(int T) {
-  const size_t ring = RM_STAGES * (size_t)((T + 7) / 8) * pair_group(pair_chunk(T)), tiles = (size_t)RM_THREADS * 64;
-  return (ring > tiles ? ring : tiles) * sizeof(float);
-}
 
 __device__ __forceinline__ void cp16(float* dst, const float* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
                : "memory");
 }
 
-__device__ __forceinline__ uint32_t cluster_rank() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-  return r;
-}
-__device__ __forceinline__ void cluster_barrier() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-__device__ __forceinline__ float ld_cluster(const float* p, uint32_t rank) {
-  uint32_t a;
-  float v;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
-  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
-  return v;
-}
-
-// One cluster of CL blocks per (b, r); block `rank` sums the chunks
-// [rank nch / CL, (rank + 1) nch / CL).  The T x T matrix of pair statistics is
-// symmetric: tile (i, j), i <= j < Tq = ceil(T / 8), holds the pairs of rows
-// t = 8 i + a and t' = 8 j + c (a, c < 8).  With `tiles` = Tq (Tq + 1) / 2 the
-// block's threads are cut into groups of `tiles`; group g takes the chunk's
-// 16-byte columns g, g + groups, ...
-// Bound by latency at 12 warps per SM (the tiles' registers) and by the shared
-// loads.  Mean absolute difference, 24 units x 16 samples x 100 steps x 4,096
-// entries: 1,463 -> 880 us against the full matrix in 4 x 4 tiles, one block
-// per (b, r).  The sorted rows alone take it: the maps of the other metrics
-// keep each pair's sum in entry order (ordered_pair_kernel).
-// rows: row t of (b, r) starts at base + ((t * U + b) * N + r) * n
-template <int CH>
-__global__ void __launch_bounds__(RM_THREADS, 2) sorted_pair_kernel(const float* rows, int T, int U, int N, int n, int CL,
-                                                                    float* dr /* [U][N][T] */) {
-  constexpr int GROUP = pair_group(CH), COLS = CH / 4, RPP = RM_THREADS / COLS;   // rows per load pass
-  static_assert(RM_THREADS % COLS == 0, "a thread loads one 16-byte column of every row it takes");
-  extern __shared__ __align__(16) float rm_smem[];
-  const uint32_t rank = CL > 1 ? cluster_rank() : 0u;
-  const int unit = blockIdx.x / CL, b = unit / N, r = unit % N;
-  const int Tq = (T + 7) / 8, tiles = Tq * (Tq + 1) / 2;
-  const int groups = min(RM_THREADS / tiles, COLS);
-  const int grp = threadIdx.x / tiles;
-  int ti = 0, tj = threadIdx.x - grp * tiles;           // tile number -> (i, j), row i of the triangle holds Tq - i tiles
-  while (tj >= Tq - ti) {
-    tj -= Tq - ti;
-    ++ti;
-  }
-  tj += ti;
-  float acc[8][8];
-#pragma unroll
-  for (int a = 0; a < 8; ++a)
-#pragma unroll
-    for (int c = 0; c < 8; ++c) acc[a][c] = 0.f;
-  // chunk c of every row -> buffer c % RM_STAGES: 16-byte asynchronous copies
-  // when the rows are a multiple of 4 entries and start on 16 bytes, plain
-  // loads otherwise (zero-padded tail)
-  const int nch = (n + CH - 1) / CH;
-  const int cb = (int)((long long)nch * rank / CL), ce = (int)((long long)nch * (rank + 1) / CL);
-  const bool vec = (n & 3) == 0 && (reinterpret_cast<uintptr_t>(rows) & 15) == 0;
-  const int lk = 4 * (threadIdx.x % COLS), lt = threadIdx.x / COLS;
-  const long long step = (long long)U * N * n;          // floats between rows t and t + 1
-  const float* lsrc = rows + lt * step + ((long long)b * N + r) * n + lk;
-  auto load_chunk = [&](int c) {
-    if (c < ce) {
-      float* xs = rm_smem + (c % RM_STAGES) * Tq * GROUP + lk;
-      const int w = n - c * CH - lk;                    // entries of the row from this column on
-      const float* src = lsrc + (long long)c * CH;
-      for (int t = lt; t < T; t += RPP, src += RPP * step) {
-        float* dst = xs + (t >> 3) * GROUP + (t & 7) * CH;
-        if (w > 3 && vec) {
-          cp16(dst, src);
-        } else {
-          float4 f = make_float4(0.f, 0.f, 0.f, 0.f);
-          if (w > 0) f.x = src[0];
-          if (w > 1) f.y = src[1];
-          if (w > 2) f.z = src[2];
-          if (w > 3) f.w = src[3];
-          *reinterpret_cast<float4*>(dst) = f;
-        }
-      }
-    }
-    asm volatile("cp.async.commit_group;" ::: "memory");
-  };
-  // Two entries at a time, the halves of a 16-byte column in swapped order for
-  // j >= 8: row groups j and j + 8 start in the same bank.  (The results of rows
-  // beyond T, whatever their buffers hold, are dropped.)
-  const int h0 = (tj >> 3 & 1) * 2;
-  for (int s = 0; s < RM_STAGES - 1; ++s) load_chunk(cb + s);
-  for (int c = cb; c < ce; ++c) {
-    asm volatile("cp.async.wait_group %0;" ::"n"(RM_STAGES - 2) : "memory");
-    __syncthreads();                                    // chunk c is there, chunk c - 1 has been read
-    load_chunk(c + RM_STAGES - 1);
-    if (grp < groups) {
-      const float* xs = rm_smem + (c % RM_STAGES) * Tq * GROUP;
-#pragma unroll 1
-      for (int k = 8 * grp; k < 2 * CH; k += 4) {       // k / 8: the column, k & 4: the second of its halves
-        const float* xr = xs + ti * GROUP + (k >> 3) * 4 + (h0 ^ (k >> 1 & 2));
-        const float* yr = xs + tj * GROUP + (k >> 3) * 4 + (h0 ^ (k >> 1 & 2));
-        float2 y[8];
-#pragma unroll
-        for (int q = 0; q < 8; ++q) y[q] = *reinterpret_cast<const float2*>(yr + q * CH);
-#pragma unroll
-        for (int a = 0; a < 8; ++a) {
-          const float2 x = *reinterpret_cast<const float2*>(xr + a * CH);
-#pragma unroll
-          for (int q = 0; q < 8; ++q) {
-            acc[a][q] += fabsf(x.x - y[q].x);
-            acc[a][q] += fabsf(x.y - y[q].y);
-          }
-        }
-        if (k & 4) k += 8 * (groups - 1);
-      }
-    }
-  }
-  asm volatile("cp.async.wait_group 0;" ::: "memory");
-  __syncthreads();
-  // the groups' tiles side by side, then summed in group order into group 0's:
-  // entry e = 8 a + c of tile q ends in rm_smem[e * RM_THREADS + q]
-  if (grp < groups) {
-#pragma unroll
-    for (int a = 0; a < 8; ++a)
-#pragma unroll
-      for (int c = 0; c < 8; ++c) rm_smem[(8 * a + c) * RM_THREADS + threadIdx.x] = acc[a][c];
-  }
-  __syncthreads();
-  if (groups > 1) {
-    for (int i = threadIdx.x; i < tiles * 64; i += RM_THREADS) {
-      float* q = rm_smem + (i / tiles) * RM_THREADS + i % tiles;
-      float v = q[0];
-      for (int g = 1; g < groups; ++g) v += q[g * tiles];
-      q[0] = v;
-    }
-    __syncthreads();
-  }
-  // this block's rows of the map: a warp per row, the blocks' partial sums in rank order
-  if (CL > 1) cluster_barrier();
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  auto total = [&](int t, int t2) {
-    int i = t >> 3, j = t2 >> 3, a = t & 7, c = t2 & 7;
-    if (i > j) {
-      const int m = i, o = a;
-      i = j;
-      j = m;
-      a = c;
-      c = o;
-    }
-    const float* q = rm_smem + (8 * a + c) * RM_THREADS + i * Tq - i * (i - 1) / 2 + (j - i);
-    if (CL == 1) return *q;
-    float v = 0.f;
-    for (int k = 0; k < CL; ++k) v += ld_cluster(q, k);
-    return v;
-  };
-  for (int t = rank + CL * warp; t < T; t += CL * (RM_THREADS / 32)) {
-    float s = 0.f;
-    for (int t2 = lane; t2 < T; t2 += 32)
-      if (t2 != t) s += total(t, t2) / (float)n;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) dr[((long long)b * N + r) * T + t] = s / (float)(T - 1);
-  }
-  if (CL > 1) cluster_barrier();                        // the peers may still read this block's tiles
-}
-
-// Cosine, mean square and mean absolute difference: one block per (b, r).
+// Cosine, mean square and mean absolute difference (of sorted rows:
+// Wasserstein-1): one block per (b, r).
 // Every pair's sum runs over the entries in index order, and every row's over
 // the steps in order, so that the map is a fixed function of the trace whatever
 // the tiling: a guided draw takes a 64-bit remainder by the sum of the weights,
@@ -236,7 +60,9 @@ __global__ void __launch_bounds__(RM_THREADS, 2) sorted_pair_kernel(const float*
 // Bound by FP32 issue and the shared loads.  Cosine map of 24 units x 16 samples
 // x 100 steps x 4,096 entries: 1,279 us as the full matrix in 4 x 4 tiles ->
 // 665 us in 8 x 8 packed tiles with the entries cut over blocks (which changed
-// the sums) -> 580 us.
+// the sums) -> 580 us.  Wasserstein-1 of 24 units x 4 samples x 100 steps x 4,096
+// entries, sort included: 735 us, and 632 with the entries cut over a cluster of
+// blocks, whose sums depended on how many maps shared the call.
 constexpr int OP_CH = 32, OP_STAGES = 4, OP_GROUP = 4 * OP_CH + 4;
 
 __host__ __device__ constexpr int op_groups(int T) { return (T + 7) / 8 * 2; }   // groups of four rows
@@ -605,27 +431,6 @@ __global__ void __launch_bounds__(GS_THREADS) guided_kernel(const float* d, int 
   for (int i = threadIdx.x; i < cells; i += GS_THREADS) S[(long long)p * cells + i] = taken[i];
 }
 
-template <int CH>
-cudaError_t launch_sorted_pair(const float* rows, int T, int U, int N, int n, int CL, float* dr, cudaStream_t st) {
-  const int sm = (int)pair_smem(T);
-  const cudaError_t e = cudaFuncSetAttribute(sorted_pair_kernel<CH>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)pair_smem(CH == 64 ? RM_MAX_T : 32));
-  if (e != cudaSuccess) return e;
-  cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = CL;
-  at[0].val.clusterDim.y = 1;
-  at[0].val.clusterDim.z = 1;
-  cfg.gridDim = dim3((unsigned)(U * N * CL));
-  cfg.blockDim = dim3(RM_THREADS);
-  cfg.dynamicSmemBytes = sm;
-  cfg.stream = st;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, sorted_pair_kernel<CH>, rows, T, U, N, n, CL, dr);
-}
-
 template <int METRIC, int RA, int CB>
 cudaError_t launch_ordered_pair_as(const float* rows, int T, int U, int N, int n, float* dr, cudaStream_t st) {
   const cudaError_t e = cudaFuncSetAttribute(ordered_pair_kernel<METRIC, RA, CB>,
@@ -678,19 +483,11 @@ cudaError_t launch_redundancy(const float* trace, int T, int U, int N, int n, in
     if (e != cudaSuccess) return e;
     rows = sorted;
   }
-  // sorted rows: blocks per (b, r), enough for several rounds over the chip's
-  // 304 resident blocks (an even last round), at least four chunks each
-  int CL = 1;
-  const int nch = (n + pair_chunk(T) - 1) / pair_chunk(T);
-  while (CL < 8 && (long long)U * N * CL < 1216 && nch >= 4 * CL) CL *= 2;
   cudaError_t e = cudaSuccess;
   switch (metric) {
     case M_COS: e = launch_ordered_pair<M_COS>(rows, T, U, N, n, dr, st); break;
     case M_MSE: e = launch_ordered_pair<M_MSE>(rows, T, U, N, n, dr, st); break;
-    case M_L1: e = launch_ordered_pair<M_L1>(rows, T, U, N, n, dr, st); break;
-    default:
-      e = pair_chunk(T) == 64 ? launch_sorted_pair<64>(rows, T, U, N, n, CL, dr, st)
-                              : launch_sorted_pair<256>(rows, T, U, N, n, CL, dr, st);
+    default: e = launch_ordered_pair<M_L1>(rows, T, U, N, n, dr, st);   // (w1: of the sorted rows)
   }
   if (e != cudaSuccess) return e;
   mean_kernel<<<(U * T + 255) / 256, 256, 0, st>>>(dr, T, U, N, d);

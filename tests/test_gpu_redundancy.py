@@ -151,11 +151,45 @@ def test_map_w1_keeps_nan_and_inf(torch, B):
     assert np.all(np.isnan(got[0])) and np.all(np.isinf(got[1])) and np.all(np.isfinite(got[2]))
 
 
-@pytest.mark.parametrize("metric", ["cosine", "mse", "l1"])
-@pytest.mark.parametrize("T,n", [(2, 3), (7, 64), (8, 256), (9, 260), (32, 516), (33, 130), (100, 1028), (128, 333)])
+def _entry_order_l1(trace):
+    """The mean-absolute-difference map in fp32, every sum in index order:
+    a pair's over the entries, a row's over the steps, the mean over the samples."""
+    T, U, N, n = trace.shape
+    d = np.zeros((U, T), np.float32)
+    for r in range(N):
+        x = trace[:, :, r]                                          # [T][U][n]
+        g = np.zeros((T, T, U), np.float32)
+        for k in range(n):
+            g += np.abs(x[:, None, :, k] - x[None, :, :, k])
+        g /= np.float32(n)
+        s = np.zeros((T, U), np.float32)
+        for t2 in range(T):
+            s += np.where(np.arange(T)[:, None] == t2, np.float32(0), g[:, t2])
+        d += (s / np.float32(T - 1)).T
+    return d / np.float32(N)
+
+
+@pytest.mark.parametrize("T,n", [(2, 64), (8, 256), (32, 128), (33, 256), (64, 512), (65, 256), (100, 1024), (128, 256)])
+def test_map_w1_bits_in_entry_order(torch, B, T, n):
+    # a map that differs in its last bits draws other guided schedules: the sorted
+    # rows' sums run in entry order in every tile shape, and a unit's map does not
+    # depend on which units share the call
+    rng = np.random.default_rng(T + n)
+    trace = rng.standard_normal((T, 4, 2, n)).astype(np.float32)
+    got = B.redundancy_map(torch.from_numpy(trace).cuda(), "w1").cpu().numpy()
+    assert np.array_equal(got, _entry_order_l1(np.sort(trace, axis=-1)))
+    one = B.redundancy_map(torch.from_numpy(np.ascontiguousarray(trace[:, 1:2])).cuda(), "w1").cpu().numpy()
+    assert np.array_equal(one[0], got[1])
+
+
+@pytest.mark.parametrize("metric", ["cosine", "mse", "l1", "w1"])
+@pytest.mark.parametrize("T,n", [(2, 3), (7, 64), (8, 256), (9, 260), (32, 516), (33, 130), (64, 64), (65, 77), (100, 1028),
+                                 (128, 333)])
 def test_map_tile_edges(torch, B, metric, T, n):
-    # row groups of eight (one, a partial one, sixteen), both chunk lengths, a ragged
-    # last chunk, several blocks per map (1,028 entries) and one
+    # the three tile shapes and the step counts where they change (32 | 33, 64 | 65), row
+    # groups of four filled in part, one chunk of 32 entries and several, a ragged last one
+    if metric == "w1":
+        n = 1 << (n - 1).bit_length()                               # the sorted rows' lengths
     rng = np.random.default_rng(T * 1000 + n)
     U, N = 2, 2
     base = rng.standard_normal((U, N, n))
