@@ -405,8 +405,10 @@ __global__ void __launch_bounds__(GS_THREADS) guided_kernel(const float* d, int 
       }
       const unsigned long long target = rk % total;
       const int run = __ffs(__ballot_sync(0xffffffffu, incl > target)) - 1;
-      const unsigned long long before = __shfl_sync(0xffffffffu, incl, run > 0 ? run - 1 : 0);
-      const unsigned long long rest = target - (run > 0 ? before : 0ull);
+      // sum of the runs in front; the comparison below adds to it, so that sums that
+      // wrap around (large eps and gamma) pick what a plain running sum picks
+      const unsigned long long front = __shfl_sync(0xffffffffu, incl, run > 0 ? run - 1 : 0);
+      const unsigned long long before = run > 0 ? front : 0ull;
       const int c0 = run * ch, cn = min(ch, cells - c0);
       int sel = -1;
       unsigned long long mine[4];                       // this lane's cells of the run: lane, lane + 32, ...
@@ -414,7 +416,7 @@ __global__ void __launch_bounds__(GS_THREADS) guided_kernel(const float* d, int 
       for (int j = 0; j < 4; ++j) mine[j] = lane + 32 * j < cn ? pre[c0 + lane + 32 * j] : 0ull;
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        const unsigned hit = __ballot_sync(0xffffffffu, lane + 32 * j < cn && mine[j] > rest);
+        const unsigned hit = __ballot_sync(0xffffffffu, lane + 32 * j < cn && before + mine[j] > target);
         if (sel < 0 && hit) sel = 32 * j + __ffs(hit) - 1;
       }
       const unsigned long long w = pre[c0 + sel] - (sel > 0 ? pre[c0 + sel - 1] : 0ull);

@@ -128,6 +128,39 @@ def test_guided_schedules_run_edges(torch, B, units, steps, K):
     assert np.array_equal(got, O.guided_schedules(d, K, 0.05, 2, rnd))
 
 
+def _wrapping_draws(q, K, rnd):
+    """Draws on 64-bit sums that wrap: the first of 32 runs of cells whose last running
+    sum exceeds the target, in it the first cell whose running sum does."""
+    M = 1 << 64
+    ch = (len(q) + 31) // 32
+    left = [int(v) for v in q]
+    out = np.zeros(len(q), np.uint8)
+    for k in range(K):
+        run, sums = 0, []
+        for v in left:
+            run = (run + v) % M
+            sums.append(run)
+        target = int(rnd[k]) % sums[-1]
+        lo = next(i for i in range(0, len(q), ch) if sums[min(i + ch, len(q)) - 1] > target)
+        pick = next(i for i in range(lo, lo + ch) if sums[i] > target)
+        out[pick], left[pick] = 1, 0
+    return out
+
+
+@pytest.mark.parametrize("eps,gamma", [(10.0, 4), (30.0, 4), (45.0, 4), (7.0, 7)])
+def test_guided_schedules_wrapping_sums(torch, B, eps, gamma):
+    # 2,400 weights whose sum passes 2^64, in the last three the sum of every run of 75 cells too
+    d = synth.dissimilarity_map(24, 100, 5).astype(np.float32)
+    q = O.guided_weights(d, eps, gamma)
+    assert sum(int(v) for v in q) > 1 << 64
+    P, K = 8, 60
+    rnd = synth.guided_randoms(P, K, 17)
+    got = B.guided_schedules(torch.from_numpy(d).cuda(), K, torch.from_numpy(rnd.view(np.int64)).cuda(), eps,
+                             gamma).cpu().numpy()
+    want = np.stack([_wrapping_draws(q, K, rnd[p]).reshape(d.shape) for p in range(P)])
+    assert np.array_equal(got, want)
+
+
 @pytest.mark.parametrize("n", [64, 128, 256, 512, 1024, 2048, 4096, 8192, 16384])
 def test_map_w1_row_lengths(torch, B, n):
     # every register-sort size (several rows per block and one) and the shared-memory sort below them;
