@@ -452,8 +452,12 @@ cudaError_t launch_ordered_pair(const float* rows, int T, int U, int N, int n, f
 
 }  // namespace
 
+// floats of the per-sample maps at the start of the scratch, a multiple of 16
+// bytes: the sorted rows behind them are read by 16-byte copies
+static size_t map_floats(int T, int U, int N) { return ((size_t)U * N * T + 3) & ~size_t(3); }
+
 size_t redundancy_scratch_bytes(int T, int U, int N, int n, int metric) {
-  size_t b = (size_t)U * N * T * sizeof(float);
+  size_t b = map_floats(T, U, N) * sizeof(float);
   if (metric == M_W1) b += (size_t)T * U * N * n * sizeof(float);
   return b;
 }
@@ -469,7 +473,7 @@ cudaError_t launch_redundancy(const float* trace, int T, int U, int N, int n, in
   float* dr = static_cast<float*>(scratch);
   const float* rows = trace;
   if (metric == M_W1) {
-    float* sorted = dr + (size_t)U * N * T;
+    float* sorted = dr + map_floats(T, U, N);
     const long long n_rows = (long long)T * U * N;
     cudaError_t e = cudaSuccess;
     switch (n) {

@@ -127,3 +127,11 @@ def test_binding_rejects_non_contiguous_buffers(B):
     with pytest.raises(ValueError):
         B._ptr(t.t())
     assert B._ptr(t) == t.data_ptr()
+
+
+@pytest.mark.parametrize("T,U,N", [(7, 3, 1), (25, 9, 1), (2, 1, 1), (100, 24, 4)])
+def test_w1_scratch_keeps_sorted_rows_on_16_bytes(B, T, U, N):
+    # the sorted rows follow the per-sample maps in the scratch
+    n = 256
+    lead = B.load().evo_redundancy_scratch_bytes(T, U, N, n, B.METRICS["w1"]) - 4 * T * U * N * n
+    assert lead % 16 == 0 and 4 * T * U * N <= lead < 4 * T * U * N + 16

@@ -232,8 +232,26 @@ def test_map_tile_edges(torch, B, metric, T, n):
 
 
 def test_map_w1_odd_number_of_maps(torch, B):
-    # 7 x 3 x 1 per-sample values in front of the sorted rows: they start off a 16-byte boundary
+    # 7 x 3 x 1 per-sample values in front of the sorted rows
     rng = np.random.default_rng(5)
     trace = rng.standard_normal((7, 3, 1, 512)).astype(np.float32)
     got = B.redundancy_map(torch.from_numpy(trace).cuda(), "w1").cpu().numpy()
     _close(got, O.redundancy_map(trace.transpose(2, 1, 0, 3).astype(np.float64), "w1"))
+
+
+@pytest.mark.parametrize("metric", ["cosine", "mse", "l1", "w1"])
+def test_map_rows_off_16_bytes(torch, B, metric):
+    # a trace and a scratch of the caller's that start 4 bytes off: the rows are read by plain loads
+    rng = np.random.default_rng(6)
+    T, U, N, n = 40, 3, 1, 256
+    trace = rng.standard_normal((T, U, N, n)).astype(np.float32)
+    m = B.METRICS[metric]
+    nb = B.load().evo_redundancy_scratch_bytes(T, U, N, n, m)
+    buf = torch.empty(trace.size + 1, device="cuda")
+    buf[1:] = torch.from_numpy(trace).cuda().flatten()
+    scratch = torch.empty(nb // 4 + 1, device="cuda")
+    d = torch.empty((U, T), device="cuda")
+    assert B.load().evo_redundancy_map(buf[1:].data_ptr(), T, U, N, n, m, d.data_ptr(), scratch[1:].data_ptr(),
+                                       torch.cuda.current_stream().cuda_stream) == B.OK
+    want = B.redundancy_map(torch.from_numpy(trace).cuda(), metric)
+    assert torch.equal(d, want)
