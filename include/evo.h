@@ -207,8 +207,9 @@ evo_status evo_denoise_noalloc(evo_handle* h, const float* obs, const float* noi
  * block (no cluster, no asynchronous copy, no tensor memory) waits on a
  * barrier that nothing arrives at, through the same wait helper as the
  * denoising-loop kernel (helper 0, limit in SM cycles, 1..10^7) or the
- * tensor-core kernels (helper 1, limit in polls, 1..10^5), so the wait runs
- * out.  Afterwards evo_get_status() returns EVO_ERR_TIMEOUT once (and clears
+ * tensor-core kernels (helper 1: the GEMMs' wait, limit in polls, 1..10^5; then
+ * the tile kernel's, the same limit in cycles, which also ends the block's later
+ * waits), so the wait runs out.  Afterwards evo_get_status() returns EVO_ERR_TIMEOUT once (and clears
  * it); the handle stays usable.  EVO_ERR_ARG for other helpers or limits. */
 evo_status evo_test_wait_timeout(evo_handle* h, int32_t helper, int64_t limit, void* stream);
 

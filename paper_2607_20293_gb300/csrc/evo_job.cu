@@ -460,7 +460,10 @@ cudaError_t launch_obs_cond(const float* w, const int* wo_dev, const int* wo, co
 // Diagnostic of the device-side failure path: one thread waits on an mbarrier
 // that nothing arrives at, through the same bounded-wait helper the loop kernel
 // (helper 0) or the tensor-core kernels (helper 1) use.  No cluster, no copy and
-// no tensor memory are involved, so giving up leaves nothing in flight.
+// no tensor memory are involved, so giving up leaves nothing in flight.  Helper 1
+// runs both of theirs, the GEMMs' and the tile kernel's, and the latter once more
+// with a limit of 10^9 cycles, which has to find the block given up and return at
+// once; the timeout is recorded if all of them ended as they should.
 __global__ void wait_probe_kernel(int helper, long long limit, int* status) {
   __shared__ uint64_t bar;
   if (threadIdx.x == 0) {
@@ -475,7 +478,18 @@ __global__ void wait_probe_kernel(int helper, long long limit, int* status) {
       cx.wait_limit = limit;
       wait_parity(smem_u32(&bar), 0u, false, cx, status);
     } else {
-      tc::mbar_wait(&bar, 0u, status, limit);
+      __shared__ int dead;
+      __shared__ int rec[3];
+      dead = rec[0] = rec[1] = rec[2] = 0;
+      tc::mbar_wait(&bar, 0u, &rec[0], limit);
+      tc::mbar_wait_live(smem_u32(&bar), 0u, &rec[1], limit, smem_u32(&dead));
+      const bool given_up = tc::block_dead(smem_u32(&dead));
+      const long long t0 = clock64();
+      tc::mbar_wait_live(smem_u32(&bar), 0u, &rec[2], 1000000000ll, smem_u32(&dead));
+      const bool at_once = clock64() - t0 < 100000000ll;
+      if (atomicOr(&rec[0], 0) == ST_TIMEOUT && atomicOr(&rec[1], 0) == ST_TIMEOUT && atomicOr(&rec[2], 0) == 0 &&
+          given_up && at_once)
+        atomicOr(status, ST_TIMEOUT);
     }
   }
 }

@@ -118,6 +118,29 @@ __device__ __forceinline__ void mbar_wait(uint64_t* bar, uint32_t parity, int* s
   atomicOr(status, ST_TIMEOUT);
 }
 
+// The wait of a kernel that runs a whole loop in one block: bounded in SM cycles,
+// and over for the whole block once one wait was in vain.  `dead` is a word of
+// shared memory, zero at the start: the wait that gives up sets it (and records
+// ST_TIMEOUT), and every later wait returns as soon as it finds it set, instead
+// of each waiting out every barrier that is left.
+__device__ __forceinline__ bool block_dead(uint32_t dead) {
+  int d;
+  asm volatile("ld.volatile.shared::cta.b32 %0, [%1];" : "=r"(d) : "r"(dead) : "memory");
+  return d != 0;
+}
+__device__ __forceinline__ void mbar_wait_live(uint32_t bar, uint32_t parity, int* status, long long limit,
+                                               uint32_t dead) {
+  if (mbar_test(bar, parity)) return;
+  const long long t0 = clock64();
+  while (!block_dead(dead)) {
+    if (mbar_test(bar, parity)) return;
+    if (clock64() - t0 > limit) {
+      asm volatile("st.volatile.shared::cta.b32 [%0], 1;" ::"r"(dead) : "memory");
+      atomicOr(status, ST_TIMEOUT);
+    }
+  }
+}
+
 __device__ __forceinline__ void mbar_arrive1(uint64_t* bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(su32(bar)) : "memory");
 }

@@ -54,7 +54,11 @@
 //
 // Warps 0-7 compute, warp 8 streams weights, warp 9 issues the MMAs (10 and 11
 // only complete the third warpgroup, which gives its registers away).  Every
-// wait on an mbarrier is bounded (evo_tc.cuh).
+// wait on an mbarrier is bounded, and once one was in vain none waits any more
+// (mbar_wait_live, evo_tc.cuh): no copy is issued from then on, the copying and
+// the issuing warp leave after their unit, and the compute warps, which meet at
+// barriers of their own, leave together at the next step's end.  What is computed
+// until then stays in bounds and is worthless; the status word says so.
 
 #include <algorithm>
 #include <cmath>
@@ -127,6 +131,15 @@ struct TileParams {
 };
 
 __device__ __forceinline__ void bar_compute() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
+// the same; true in every thread if x is in one
+__device__ __forceinline__ bool bar_compute_any(bool x) {
+  uint32_t r;
+  asm volatile("{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n bar.red.or.pred q, 1, 256, p;\n selp.u32 %0, 1, 0, q;\n}\n"
+               : "=r"(r)
+               : "r"((uint32_t)x)
+               : "memory");
+  return r != 0;
+}
 
 __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
   asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
@@ -140,12 +153,8 @@ __device__ __forceinline__ void commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
 __device__ __forceinline__ uint64_t desc64(uint32_t lo, uint32_t hi) { return ((uint64_t)hi << 32) | lo; }
-__device__ __noinline__ void wait_slow(uint32_t bar, uint32_t parity, int* status, long long limit) {
-  for (long long i = 0; i < limit; ++i) {
-    if (mbar_test(bar, parity)) return;
-    if (i > 64) __nanosleep(32);
-  }
-  atomicOr(status, ST_TIMEOUT);
+__device__ __noinline__ void wait_slow(uint32_t bar, uint32_t parity, int* status, long long limit, uint32_t dead) {
+  mbar_wait_live(bar, parity, status, limit, dead);
 }
 
 // 16 rows x 32 (64) fp32 columns in the layout of mma.sync accumulators: tile j
@@ -269,6 +278,7 @@ struct Bars {
   uint64_t hready[2], hempty[2];          // second-GEMM operand buffers: written (8 warps) / consumed (commit)
   uint64_t rfull;                         // R finished (commit)
   uint32_t tslot;
+  uint32_t dead;                          // a wait was in vain
 };
 
 // mean and 1/std of the lane's two rows (64 columns each, the rest in the quad's
@@ -385,6 +395,7 @@ __global__ void __launch_bounds__(TTHREADS, 1) tile_kernel(const TileParams p) {
       mbar_init1(&B->hempty[i], 1);
     }
     mbar_init1(&B->rfull, 1);
+    B->dead = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
@@ -401,7 +412,8 @@ __global__ void __launch_bounds__(TTHREADS, 1) tile_kernel(const TileParams p) {
     // descriptor words, leave a wait that does not pass at once to a call, and
     // run uniformly over the warp with one elected lane issuing (1,000 samples at
     // full refresh: 39.4 ms with one lane in a divergent branch, 35.0).
-    const uint32_t bfull = su32(B->full), bempty = su32(B->empty);
+    const uint32_t bfull = su32(B->full), bempty = su32(B->empty), dead = su32(&B->dead);
+    bool leave = false;                                // the block gives up (uniform)
     uint32_t s = 0, ph = 0;                            // ring slot, its phase
     auto next_slot = [&]() {
       if (++s == NSLOTS) {
@@ -410,24 +422,24 @@ __global__ void __launch_bounds__(TTHREADS, 1) tile_kernel(const TileParams p) {
       }
     };
     auto wait = [&](uint32_t bar, uint32_t parity) {
-      if (!mbar_test(bar, parity)) wait_slow(bar, parity, p.status, p.wait_limit);
+      if (!mbar_test(bar, parity)) wait_slow(bar, parity, p.status, p.wait_limit, dead);
     };
     if (warp == 8) {
       // ------------------------------------------------ weights and vectors: bulk copies
       const uint32_t bvfull = su32(B->vfull), bvempty = su32(B->vempty), dring = su32(ring), dvec = su32(vecs);
       uint32_t units = 0;
-      for (int j = blockIdx.x; j < p.n_jobs; j += gridDim.x) {
+      for (int j = blockIdx.x; j < p.n_jobs && !leave; j += gridDim.x) {
         const uint64_t* mk = p.mask + (long long)lattice_of(p, j) * p.T * 2;
         uint64_t nxt = __ldg(mk);
-        for (int t = 0; t < p.T; ++t) {
+        for (int t = 0; t < p.T && !leave; ++t) {
           uint64_t m = uniform64(nxt);
           if (t + 1 < p.T) nxt = __ldg(mk + 2 * (t + 1));
-          while (m) {
+          while (m && !leave) {
             const int b = __ffsll((long long)m) - 1, l = b / 3, u = b - 3 * l;
             m &= m - 1;
             const uint32_t vb = units & 1;
             wait(bvempty + 8 * vb, ((units >> 1) & 1u) ^ 1u);
-            if (elect_one()) {
+            if (elect_one() && !block_dead(dead)) {
               expect_tx(bvfull + 8 * vb, vec_floats(u) * 4);
               bulk_load(dvec + vb * VEC_BYTES, p.vec + (long long)l * VEC_LAYER + vec_off(u), vec_floats(u) * 4,
                         bvfull + 8 * vb);
@@ -438,12 +450,13 @@ __global__ void __launch_bounds__(TTHREADS, 1) tile_kernel(const TileParams p) {
 #pragma unroll 1
             for (; src != end; src += SLOT) {
               wait(bempty + 8 * s, ph ^ 1u);
-              if (elect_one()) {
+              if (elect_one() && !block_dead(dead)) {
                 expect_tx(bfull + 8 * s, SLOT);
                 bulk_load(dring + s * SLOT, src, SLOT, bfull + 8 * s);
               }
               next_slot();
             }
+            leave = __any_sync(0xffffffffu, block_dead(dead));
           }
         }
       }
@@ -457,13 +470,13 @@ __global__ void __launch_bounds__(TTHREADS, 1) tile_kernel(const TileParams p) {
       const uint32_t baf = su32(B->afull), bae = su32(B->aempty), bhr = su32(B->hready), bhe = su32(B->hempty);
       const uint32_t bx = su32(&B->xready), brf = su32(&B->rfull);
       uint32_t units = 0, na = 0, nh = 0;               // phases: units, first-GEMM chunks; second-GEMM chunks / 2
-      for (int j = blockIdx.x; j < p.n_jobs; j += gridDim.x) {
+      for (int j = blockIdx.x; j < p.n_jobs && !leave; j += gridDim.x) {
         const uint64_t* mk = p.mask + (long long)lattice_of(p, j) * p.T * 2;
         uint64_t nxt = __ldg(mk);
-        for (int t = 0; t < p.T; ++t) {
+        for (int t = 0; t < p.T && !leave; ++t) {
           uint64_t m = uniform64(nxt);
           if (t + 1 < p.T) nxt = __ldg(mk + 2 * (t + 1));
-          while (m) {
+          while (m && !leave) {
             const int b = __ffsll((long long)m) - 1, u = b % 3;
             m &= m - 1;
             wait(bx, units & 1u);
@@ -535,6 +548,7 @@ __global__ void __launch_bounds__(TTHREADS, 1) tile_kernel(const TileParams p) {
               }
             }
             ++units;
+            leave = __any_sync(0xffffffffu, block_dead(dead));
           }
         }
       }
@@ -549,6 +563,9 @@ __global__ void __launch_bounds__(TTHREADS, 1) tile_kernel(const TileParams p) {
     uint4* cache = p.cache + (long long)blockIdx.x * p.U * 16 * TCT + tid;
     uint32_t na = 0, nh[2] = {0, 0}, units = 0;
     float2 a[2][32];                                   // columns 8 j + 2 tq, + 1 of rows g, g + 8
+    auto wait = [&](uint64_t* bar, uint32_t parity) {
+      mbar_wait_live(su32(bar), parity, p.status, p.wait_limit, su32(&B->dead));
+    };
 
     for (int j = blockIdx.x; j < p.n_jobs; j += gridDim.x) {
       const int lat = lattice_of(p, j), part = j % p.jobs_per_lat;
@@ -565,12 +582,13 @@ __global__ void __launch_bounds__(TTHREADS, 1) tile_kernel(const TileParams p) {
       float* es = xs + 256;                                     // [16][16]: the output head's sums
 
       const float* tab = reinterpret_cast<const float*>(hid);
-      // the step-end tables -> operand buffers (free between units)
-      auto load_tab = [&]() {
-        bar_compute();                                  // nobody reads the buffers
+      // the step-end tables -> operand buffers (free between units); false: the block gives up
+      auto load_tab = [&]() -> bool {
+        if (bar_compute_any(block_dead(su32(&B->dead)))) return false;   // (nobody reads the buffers)
         for (int i = tid; i < tab_floats(p.A) / 4; i += TCT)
           asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(su32(hid + 16 * i)), "l"(p.tab + 4 * i) : "memory");
         asm volatile("cp.async.commit_group;" ::: "memory");
+        return true;
       };
       auto wait_tab = [&]() {
         asm volatile("cp.async.wait_group 0;" ::: "memory");
@@ -596,7 +614,7 @@ __global__ void __launch_bounds__(TTHREADS, 1) tile_kernel(const TileParams p) {
         }
       };
 
-      load_tab();
+      if (!load_tab()) break;
       // x <- noise[0]
       for (int c = sact; c < p.A; c += 2) {
         const float v = nz[c];
@@ -642,7 +660,7 @@ __global__ void __launch_bounds__(TTHREADS, 1) tile_kernel(const TileParams p) {
           {
             float mean[2], rstd[2];
             tile_stats(a, mean, rstd);
-            mbar_wait(&B->vfull[units & 1], (units >> 1) & 1u, p.status, p.wait_limit);
+            wait(&B->vfull[units & 1], (units >> 1) & 1u);
             const float2 nm0 = both(-mean[0]), nm1 = both(-mean[1]), rs0 = both(rstd[0]), rs1 = both(rstd[1]);
             const float2 *gv = reinterpret_cast<const float2*>(vec) + tq, *bv = gv + TE / 2;
 #pragma unroll
@@ -665,7 +683,7 @@ __global__ void __launch_bounds__(TTHREADS, 1) tile_kernel(const TileParams p) {
 
           auto wait_acc = [&]() -> uint32_t {           // the next chunk's accumulator
             const uint32_t acc = na & 1u;
-            mbar_wait(&B->afull[acc], (na >> 1) & 1u, p.status, p.wait_limit);
+            wait(&B->afull[acc], (na >> 1) & 1u);
             tc_fence_after();
             return acc;
           };
@@ -675,7 +693,7 @@ __global__ void __launch_bounds__(TTHREADS, 1) tile_kernel(const TileParams p) {
             ++na;
           };
           auto wait_hid = [&](int buf) {                // the operand buffer's previous chunk is consumed
-            mbar_wait(&B->hempty[buf], (nh[buf] & 1u) ^ 1u, p.status, p.wait_limit);
+            wait(&B->hempty[buf], (nh[buf] & 1u) ^ 1u);
             ++nh[buf];
           };
           auto put_hid = [&](int buf) {
@@ -857,7 +875,7 @@ __global__ void __launch_bounds__(TTHREADS, 1) tile_kernel(const TileParams p) {
           }
 
           // r = R + bias: a += r, c_b <- bf16(r)
-          mbar_wait(&B->rfull, units & 1u, p.status, p.wait_limit);
+          wait(&B->rfull, units & 1u);
           tc_fence_after();
           const uint32_t vb = units & 1u;
           ++units;
@@ -887,7 +905,7 @@ __global__ void __launch_bounds__(TTHREADS, 1) tile_kernel(const TileParams p) {
         }
 
         // step end: eps = LN_f(a) W_head + b_head, the sampler step, the next embedding
-        load_tab();
+        if (!load_tab()) break;
         {
           float xv[8], zv[8];                           // x and the step's noise of this lane's actions
 #pragma unroll
@@ -956,7 +974,7 @@ __global__ void __launch_bounds__(TTHREADS, 1) tile_kernel(const TileParams p) {
     }
   }
   __syncwarp();
-  settle_after_timeout(p.status, false);   // after a timeout, copies and MMAs may still be in flight
+  settle_after_timeout(p.status, block_dead(su32(&B->dead)));   // then copies and MMAs may still be in flight
   tc_fence_before();
   __syncthreads();
   if (warp == 9) tmem_dealloc(tmem, 512);
@@ -1149,7 +1167,7 @@ cudaError_t tile_run(const TileState* s, const TileCall& c) {
   p.out = c.out;
   p.scale = 0.125f;               // 1 / sqrt(64)
   p.status = c.status;
-  p.wait_limit = WAIT_POLLS_DEFAULT;
+  p.wait_limit = WAIT_CYCLES_DEFAULT;
   const int grid = std::min(p.n_jobs, s->cache_slots);
   tile_kernel<<<grid, TTHREADS, TILE_SMEM, c.st>>>(p);
   return cudaGetLastError();

@@ -5,7 +5,12 @@ form that cannot fault: evo_test_wait_timeout runs the loop kernel's and the
 tensor-core kernels' wait helpers in one thread of one block, on a barrier
 that nothing arrives at, with a tiny limit (no cluster, no copy, no tensor
 memory in flight).  The status must report the timeout once, and the next
-ordinary call must succeed and match the oracle."""
+ordinary call must succeed and match the oracle.
+
+The tensor-core probe (helper 1) reports the timeout only if the GEMMs' wait
+gave up, the tile kernel's wait gave up and marked its block, and a second wait
+of the tile kernel, with a limit of half a second, then returned at once: a
+block that runs a whole loop must not wait out every barrier that is left."""
 import numpy as np
 import pytest
 
