@@ -183,13 +183,12 @@ evo_status evo_set_profile_events(evo_handle* h, void* start, void* stop);
  * no counterpart; this is an interface choice.  Arguments, layouts and
  * results are those of evo_denoise, and it always takes the one-cluster-per-job
  * path, so its output is bit-identical to an evo_denoise call that takes that
- * path.  The per-call scratch (the observation tokens' cross-attention
+ * path (with wide_rows < 0 every evo_denoise call does).  The per-call scratch (the observation tokens' cross-attention
  * keys/values and the condition MLP's intermediates) lives in one file-scope
  * device array of 8 MiB that every GPU which loads this library holds until
  * the process exits; N * n_obs * (2 * n_layer + 6) * n_emb * 4 bytes must fit
  * in it (186 samples of the Push-T-shaped model), else EVO_ERR_SHAPE and
- * nothing is launched.  (A call that runs on the tile kernel, see wide_rows,
- * keeps them in the handle's buffers instead; the limit is the same.)  No cudaMalloc, cudaFree or allocating library routine
+ * nothing is launched.  No cudaMalloc, cudaFree or allocating library routine
  * is called.  The first call on a device looks up the array's device address
  * (cudaGetSymbolAddress) and keeps it for later calls.  All calls share the
  * array and every call overwrites all of it

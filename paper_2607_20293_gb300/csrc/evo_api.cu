@@ -1180,7 +1180,6 @@ evo_status evo_denoise_noalloc(evo_handle* h, const float* obs, const float* noi
   const int* err = nullptr;
   evo_status s = stage_schedules(h, S, 1, S_rows, false, st, &err);
   if (s != EVO_OK) return s;
-  if (use_tile(h, N)) return run_tile(h, obs, noise, out_actions, N, 1, S_rows, err, st);
   EVO_CUDA(obs_cond(h, obs, N, kv + kv_floats, kv, st));
   const Pick pk = pick_decomposition(h, N);
   JobParams p = *pk.base;

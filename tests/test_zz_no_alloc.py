@@ -84,3 +84,24 @@ def test_noalloc_size_limit(torch, B):
     want = ev.denoise(obs[:m], noise_m, S).cpu().numpy()
     assert np.array_equal(got, want)
     assert ev.status() == B.OK
+
+
+@pytest.mark.parametrize("n", [109, 128, 186])
+@pytest.mark.parametrize("frac", [0.05, 0.5])
+def test_noalloc_keeps_the_cluster_path(torch, B, n, frac):
+    # sizes at which evo_denoise of a handle with default options may run elsewhere
+    cfg = synth.config("pusht", n_steps=20)
+    W = synth.make_weights(cfg, 0)
+    S = synth.bernoulli_schedule(24, 20, frac, 13)
+    obs_h, noise_h = synth.make_obs(cfg, n, 61), synth.make_noise(cfg, n, 62)
+    obs, noise = torch.from_numpy(obs_h).cuda(), torch.from_numpy(noise_h).cuda()
+    ev = B.Evo(cfg, W, n)
+    out = torch.full((n, cfg["horizon"], cfg["action_dim"]), float("nan"), device="cuda")
+    got = ev.denoise_noalloc(obs, noise, S, out).cpu().numpy()
+    info = ev.launch_info()
+    assert ev.last_call()["path"] == "cluster" and info["cluster"] > 1
+    want = B.Evo(cfg, W, n, wide_rows=-1).denoise(obs, noise, S).cpu().numpy()
+    assert np.array_equal(got, want)
+    idx = [0, n - 1]
+    assert float(np.max(np.abs(got[idx] - O.denoise(W, cfg, obs_h[idx], noise_h[:, idx], S)))) <= TOL_BF16
+    assert ev.status() == B.OK
