@@ -79,9 +79,9 @@ typedef struct evo_config {
   int32_t wide_rows;    /* batch-wide tensor-core path for calls of at least this many action-token
                            rows (samples x horizon); 0 = the library's choice (2048 with a 4-CTA
                            decomposition, else 1024; and, with cluster and job_samples left to it
-                           too, blocks of 8 samples on their own for calls of 109 samples and more
-                           of n_emb 256, 4 heads, horizon 16); < 0 = never.  bf16 with n_emb 256
-                           or 512, head size 64, horizon 16 or 32, action dim <= 16, at most 7
+                           too, blocks of 8 samples on their own where they are faster for such
+                           calls of n_emb 256, 4 heads, horizon 16); < 0 = never.  bf16 with n_emb
+                           256 or 512, head size 64, horizon 16 or 32, action dim <= 16, at most 7
                            observation tokens */
 } evo_config;
 
@@ -115,8 +115,8 @@ evo_status evo_destroy(evo_handle* h);
  *          b = 3l + {0 SA, 1 CA, 2 FFN}) or L (row l covers the three units of layer l).
  *          A host lattice is validated before launch; a device lattice is checked on the
  *          device (EVO_ERR_SCHEDULE in the status word, outputs untouched), except on
- *          the batch-wide path, which copies it to the host (one synchronisation) and
- *          returns EVO_ERR_SCHEDULE before any launch.
+ *          in calls of wide_rows rows and more (batch-wide path, tile kernel), which copy
+ *          it to the host (one synchronisation) and return EVO_ERR_SCHEDULE before any launch.
  *   out    device [N][H][A]             final actions (normalised space, after T steps)
  */
 evo_status evo_denoise(evo_handle* h, const float* obs, const float* noise,

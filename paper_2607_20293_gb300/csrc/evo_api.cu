@@ -983,19 +983,19 @@ bool use_wide(const evo_handle* h, long long samples) {
   return h->wide && samples * h->H >= h->wide_rows && samples * h->H <= wide_rows_capacity(h->wide);
 }
 
-// The tile path serves calls of more than three rounds of the 4-CTA clusters
-// (36 fit): 108 samples of the 10-action policy at refresh fraction 0.125 / 1.0
-// take 7.1 / 34.5 ms on tiles and 7.1 / 34.1 in three rounds, four rounds 9.4 / 45.6.
-constexpr long long TILE_MIN_SAMPLES = 109;
-bool use_tile(const evo_handle* h, long long samples) { return h->tile && samples >= TILE_MIN_SAMPLES; }
-
+// The tile path serves calls that the batch-wide path would serve too: both
+// round the same values (the condition path's operands, the head's weights) to
+// bf16, where the cluster path, which takes all smaller calls, keeps them in
+// fp32.  (109 .. 127 samples of the 10-action policy at refresh fraction 0.125 /
+// 1.0 would take 7.1 / 34.5 ms on tiles and take 9.4 / 45.6 in four rounds of the
+// 36 clusters.)
 // Where the batch-wide path is the other choice, it stays ahead on one sparse
 // lattice for few samples (a tile adds the skipped units' caches 64 KiB at a
 // time on one SM): 128 / 176 / 208 samples of the 10-action policy at fraction
 // 0.05 take 3.3 / 3.6 / 3.7 ms there and 4.1 on tiles, at 0.08 5.0 / 5.5 / 5.7
 // and 5.5, at 0.125 7.1 / 7.8 / 8.1 and 7.1.
 bool sparse_for_tile(const evo_handle* h, long long samples, int S_rows) {
-  if (samples >= 224 || samples * h->H < h->wide_rows) return false;
+  if (samples >= 224) return false;
   const size_t n = (size_t)S_rows * h->T;
   size_t cells = 0;
   for (size_t i = 0; i < n; ++i) cells += h->last_sched[i];
@@ -1022,25 +1022,16 @@ bool population_on_tiles(const evo_handle* h, const uint8_t* S, int P, int N_obs
   return tile < cluster;
 }
 
-// Lattices for a tile-path call.  Calls of wide_rows rows and more are the ones
-// whose device lattices are checked before anything is launched.
-evo_status stage_tile(evo_handle* h, const uint8_t* S, int n_sched, int rows, bool add_ones, long long samples,
-                      cudaStream_t st, const int** err) {
-  *err = nullptr;
-  if (samples * h->H >= h->wide_rows) return stage_wide(h, S, n_sched, rows, add_ones, st);
-  return stage_schedules(h, S, n_sched, rows, add_ones, st, err);
-}
-
 // The tile path over n_sched staged lattices of N samples each.  More than one
 // lattice: out holds the samples of all, the last is a population's reference
 // (actions: the candidates' copy or null, dev: their deviation).
 evo_status run_tile(evo_handle* h, const float* obs, const float* noise, float* out, int N, int n_sched, int S_rows,
-                    const int* err, cudaStream_t st, float* actions = nullptr, float* dev = nullptr) {
+                    cudaStream_t st, float* actions = nullptr, float* dev = nullptr) {
   long long n = 0;
   EVO_CUDA(wide_condition(h->wide, obs, N, nullptr, true, h->status, true, st, &n));
   TileCall c{};
   EVO_CUDA(wide_masks(h->wide, h->sched, S_rows, n_sched, st, &c.mask));
-  n += 2 + (err ? 1 : 0);
+  n += 2;
   if (n_sched > 1) {                           // the longest jobs first
     EVO_CUDA(launch_order(h->sched, (long long)S_rows * h->T, n_sched, h->count, h->order, st));
     c.order = h->order;
@@ -1051,7 +1042,6 @@ evo_status run_tile(evo_handle* h, const float* obs, const float* noise, float* 
   c.kv_time = wide_tile_kv_time(h->wide);
   c.stab = h->stab;
   c.out = out;
-  c.sched_err = err;
   c.n_sched = n_sched;
   c.per_sched = N;
   c.obs_mod = N;
@@ -1080,15 +1070,10 @@ evo_status run(evo_handle* h, const float* obs, const float* noise, const uint8_
   if (N <= 0 || N > h->max_batch) return EVO_ERR_SHAPE;
   if (S_rows != h->U && S_rows != h->L) return EVO_ERR_SCHEDULE;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  if (!trace && use_tile(h, N)) {
-    const int* err = nullptr;
-    const evo_status s = stage_tile(h, S, 1, S_rows, false, N, st, &err);
-    if (s != EVO_OK) return s;
-    if (!sparse_for_tile(h, N, S_rows)) return run_tile(h, obs, noise, out, N, 1, S_rows, err, st);
-  }
   if (use_wide(h, N)) {
     const evo_status s = stage_wide(h, S, 1, S_rows, false, st);
     if (s != EVO_OK) return s;
+    if (!trace && h->tile && !sparse_for_tile(h, N, S_rows)) return run_tile(h, obs, noise, out, N, 1, S_rows, st);
     h->last_cond_kernels = 0;                  // the batch-wide sequence computes kv_obs itself
     EVO_CUDA(launch_wide(h, obs, noise, out, N, N, 1, S_rows, st, trace));
     return finish(h, st);
@@ -1215,16 +1200,9 @@ evo_status evo_denoise_population(evo_handle* h, const float* obs, const float* 
     const evo_status s = stage_wide(h, S_pop, P, S_rows, true, st);
     if (s != EVO_OK) return s;
   }
-  if (use_tile(h, samples)) {
-    const int* err = nullptr;
-    const uint8_t* lat = host_checked ? h->last_sched.data() : (is_device_ptr(S_pop) ? nullptr : S_pop);
-    if (lat && population_on_tiles(h, lat, P, N_obs, S_rows)) {
-      if (!host_checked) {
-        const evo_status s = stage_schedules(h, S_pop, P, S_rows, true, st, &err);
-        if (s != EVO_OK) return s;
-      }
-      return run_tile(h, obs, noise, h->pop_x, N_obs, P + 1, S_rows, err, st, out_actions, dev_l2);
-    }
+  if (host_checked && h->tile) {
+    if (population_on_tiles(h, h->last_sched.data(), P, N_obs, S_rows))
+      return run_tile(h, obs, noise, h->pop_x, N_obs, P + 1, S_rows, st, out_actions, dev_l2);
   } else if (host_checked) {
     h->last_cond_kernels = 0;                  // the batch-wide sequence computes kv_obs itself
     EVO_CUDA(launch_wide(h, obs, noise, h->pop_x, (int)samples, N_obs, P + 1, S_rows, st));

@@ -110,7 +110,6 @@ constexpr int LAYER_SLOTS = unit_slots(0) + unit_slots(1) + unit_slots(2);
 struct TileParams {
   int L, A, n_obs, T, U;
   int n_jobs, jobs_per_lat, per_sched, obs_mod, sampler;
-  const int* sched_err;            // nonzero: schedule invalid, do nothing
   const int* order;                // lattices in the order in which their jobs are taken, or null
   const uint64_t* mask;            // [n_sched][T][2]: units refreshed at t, units whose cache holds a value
   const uint8_t* wpack;            // [L][LAYER_SLOTS][SLOT]
@@ -378,7 +377,6 @@ __global__ void __launch_bounds__(TTHREADS, 1) tile_kernel(const TileParams p) {
   float* vecs = reinterpret_cast<float*>(ring + NSLOTS * SLOT);     // [2][VEC_BYTES / 4]
   Bars* B = reinterpret_cast<Bars*>(vecs + 2 * VEC_BYTES / 4);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (p.sched_err && *p.sched_err) return;                          // the same answer in every thread
   if (warp == 9) tmem_alloc(&B->tslot, 512);
   if (threadIdx.x == 0) {
     for (int s = 0; s < NSLOTS; ++s) {
@@ -1152,7 +1150,6 @@ cudaError_t tile_run(const TileState* s, const TileCall& c) {
   p.per_sched = c.per_sched;
   p.obs_mod = c.obs_mod;
   p.sampler = s->sampler;
-  p.sched_err = c.sched_err;
   p.mask = c.mask;
   p.order = c.order;
   p.wpack = s->wpack;

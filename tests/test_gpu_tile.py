@@ -1,6 +1,6 @@
 """GPU parity of the tile path (one block runs the whole loop of up to 8 samples)
-against the float64 oracle: the library's own choice from 109 samples on for
-n_emb 256, horizon 16.
+against the float64 oracle: the library's own choice from 128 samples (2,048
+action-token rows) on for n_emb 256, horizon 16.
 
 Cases are the edges of its tiles and operands: a last tile of 1 .. 8 samples,
 1 and 16 actions, 1 and 7 observation tokens (2 and 8 memory keys), both
@@ -45,12 +45,12 @@ def close(got, want, what=""):
     assert err <= TOL, f"{what}: max-abs {err:.3e}"
 
 
-# 109 = 13 tiles and 5 samples, 112 = 14 full tiles, 113 = a tile of one sample
+# 128 = 16 full tiles, 129 = a tile of one sample, 133 = a tile of 5, 143 = of 7
 @pytest.mark.parametrize("n,over,frac", [
-    (109, {}, 0.3),
-    (112, dict(action_dim=16, n_obs=7, obs_dim=30), 1.0),
-    (113, dict(action_dim=1, n_obs=1), 0.125),
-    (120, dict(sampler="ddim", n_layer=1), 0.5),
+    (133, {}, 0.3),
+    (128, dict(action_dim=16, n_obs=7, obs_dim=30), 1.0),
+    (129, dict(action_dim=1, n_obs=1), 0.2),
+    (143, dict(sampler="ddim", n_layer=1), 0.5),
     (230, dict(n_layer=2, action_dim=5), 0.05),
 ])
 def test_tile_matches_oracle(torch, B, n, over, frac):
@@ -105,9 +105,9 @@ def test_tile_population_edge_lattices(torch, B, empty):
 
 def test_tile_lattice_forms(torch, B):
     # coarse [L][T] and device lattices give the bits of the unit lattice on the
-    # host; an invalid device lattice is reported and leaves the output alone
+    # host; an invalid lattice is refused before anything is launched
     cfg = synth.config("pusht", n_steps=20, n_layer=2)
-    n = 110
+    n = 130
     W = synth.make_weights(cfg, 0)
     obs = torch.from_numpy(synth.make_obs(cfg, n, 91)).cuda()
     noise = torch.from_numpy(synth.make_noise(cfg, n, 92)).cuda()
@@ -120,6 +120,33 @@ def test_tile_lattice_forms(torch, B):
     bad = torch.from_numpy(S).cuda()
     bad[1, 3] = 2
     out = torch.full((n, 16, 2), 5.0, device="cuda")
-    ev.denoise(obs, noise, bad, out=out)
-    assert ev.status() == B.ERR_SCHEDULE
-    assert torch.all(out == 5.0)
+    for lattice in (bad, bad.cpu().numpy()):
+        with pytest.raises(B.EvoError) as e:
+            ev.denoise(obs, noise, lattice, out=out)
+        assert e.value.code == B.ERR_SCHEDULE
+    assert torch.all(out == 5.0) and ev.status() == B.OK
+
+
+@pytest.mark.parametrize("n", [109, 127])
+def test_calls_below_the_tile_threshold_stay_on_clusters(torch, B, n):
+    # the cluster path's condition kernels and head keep their operands in fp32:
+    # a handle with default options gives the bits of one that has no other path,
+    # for a query batch and for a population, wherever the lattices are
+    cfg = synth.config("pusht", n_steps=20, n_layer=2)
+    W = {k: (v * np.float32(1.001)).astype(np.float32) for k, v in synth.make_weights(cfg, 0).items()}   # not in bf16
+    obs = torch.from_numpy(synth.make_obs(cfg, n, 94)).cuda()
+    noise = torch.from_numpy(synth.make_noise(cfg, n, 95)).cuda()
+    S = synth.bernoulli_schedule(6, 20, 0.3, 96)
+    ev, cl = B.Evo(cfg, W, n), B.Evo(cfg, W, n, wide_rows=-1)
+    want = cl.denoise(obs, noise, S)
+    for lattice in (S, torch.from_numpy(S).cuda()):
+        assert torch.equal(ev.denoise(obs, noise, lattice), want)
+        assert ev.last_call()["path"] == "cluster" and not on_tiles(ev)
+    P = n - 1
+    pop = np.stack([synth.bernoulli_schedule(6, 20, 0.5, 200 + p) for p in range(P)])
+    o1, z1 = obs[:1].contiguous(), noise[:, :1].contiguous()
+    want, want_dev = cl.population(o1, z1, pop)
+    for lattice in (pop, torch.from_numpy(pop).cuda()):
+        x, dev = ev.population(o1, z1, lattice)
+        assert torch.equal(x, want) and torch.equal(dev, want_dev)
+        assert ev.last_call()["path"] == "cluster" and not on_tiles(ev)
