@@ -983,7 +983,13 @@ bool use_wide(const evo_handle* h, long long samples) {
   return h->wide && samples * h->H >= h->wide_rows && samples * h->H <= wide_rows_capacity(h->wide);
 }
 
-// The tile path serves calls that the batch-wide path would serve too: both
+// The tile path serves calls that the batch-wide path would serve too, every
+// population among them: a lattice's refreshed cells are work for its own tiles
+// there, and launches over all rows here.  Push-T shaped, tiles / batch-wide: 12
+// candidates x 11 observations of 5 .. 60 % density 33.7 / 49.5 ms, 127 x 1 33.9 /
+// 58.8, 16 x 16 33.7 / 53.4, 64 x 16 33.8 / 97.5.  (4-CTA clusters would take
+// 18.9 / 17.4 / 37.2 / 133, but pass the residual stream's LayerNorm input and the
+// second GEMM's partial sums on in bf16, which both of these keep in fp32.)  Both
 // round the same values (the condition path's operands, the head's weights) to
 // bf16, where the cluster path, which takes all smaller calls, keeps them in
 // fp32.  (109 .. 127 samples of the 10-action policy at refresh fraction 0.125 /
@@ -1000,26 +1006,6 @@ bool sparse_for_tile(const evo_handle* h, long long samples, int S_rows) {
   size_t cells = 0;
   for (size_t i = 0; i < n; ++i) cells += h->last_sched[i];
   return 8 * cells < n;
-}
-
-// A population's lattices differ in length, so the choice is by the estimated
-// times of both, longest first on either: a job of c refreshed cells and T steps
-// takes 8 us a step + 4.4 us a cell on a cluster of 4 (a sample each) and 23 +
-// 13.2 on a tile (up to 8 samples), the reference's being the longest.  Push-T
-// shaped, tiles / clusters: 12 candidates x 11 observations of 5 .. 60 % density
-// 33.8 / 22.0 ms, 16 x 16 33.8 / 38.6, 64 x 16 34.1 / 129.6; 119 x 1 of 100 cells
-// 34.1 / 11.4.
-bool population_on_tiles(const evo_handle* h, const uint8_t* S, int P, int N_obs, int S_rows) {
-  const evo_handle::Alt* four = h->n_alt && h->alt[h->n_alt - 1].base.C == 4 ? &h->alt[h->n_alt - 1] : nullptr;
-  if (!four) return true;
-  const size_t n = (size_t)P * S_rows * h->T;
-  const double per = S_rows == h->U ? 1.0 : 3.0, all = (double)h->U * h->T;
-  double cells = all;                                  // of the reference
-  for (size_t i = 0; i < n; ++i) cells += S[i] ? per : 0.0;
-  const double jobs = P + 1.0, tiles = (N_obs + 7) / 8;
-  const double cluster = std::max(8.0 * h->T + 4.4 * all, N_obs * (jobs * 8.0 * h->T + 4.4 * cells) / four->max_clusters);
-  const double tile = std::max(23.0 * h->T + 13.2 * all, tiles * (jobs * 23.0 * h->T + 13.2 * cells) / h->num_sms);
-  return tile < cluster;
 }
 
 // The tile path over n_sched staged lattices of N samples each.  More than one
@@ -1195,15 +1181,10 @@ evo_status evo_denoise_population(evo_handle* h, const float* obs, const float* 
   if (S_rows != h->U && S_rows != h->L) return EVO_ERR_SCHEDULE;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   const int HA = h->H * h->A;
-  const bool host_checked = use_wide(h, samples);     // such calls' device lattices are checked before any launch
-  if (host_checked) {
+  if (use_wide(h, samples)) {
     const evo_status s = stage_wide(h, S_pop, P, S_rows, true, st);
     if (s != EVO_OK) return s;
-  }
-  if (host_checked && h->tile) {
-    if (population_on_tiles(h, h->last_sched.data(), P, N_obs, S_rows))
-      return run_tile(h, obs, noise, h->pop_x, N_obs, P + 1, S_rows, st, out_actions, dev_l2);
-  } else if (host_checked) {
+    if (h->tile) return run_tile(h, obs, noise, h->pop_x, N_obs, P + 1, S_rows, st, out_actions, dev_l2);
     h->last_cond_kernels = 0;                  // the batch-wide sequence computes kv_obs itself
     EVO_CUDA(launch_wide(h, obs, noise, h->pop_x, (int)samples, N_obs, P + 1, S_rows, st));
     EVO_CUDA(launch_pop_dev(h->pop_x, P, N_obs, HA, dev_l2, st));
@@ -1213,10 +1194,8 @@ evo_status evo_denoise_population(evo_handle* h, const float* obs, const float* 
     return finish(h, st);
   }
   const int* err = nullptr;
-  if (!host_checked) {
-    const evo_status s = stage_schedules(h, S_pop, P, S_rows, true, st, &err);
-    if (s != EVO_OK) return s;
-  }
+  evo_status s = stage_schedules(h, S_pop, P, S_rows, true, st, &err);
+  if (s != EVO_OK) return s;
   EVO_CUDA(obs_cond(h, obs, N_obs, h->cond_scratch, h->kv_obs, st));
   Pick pk = pick_decomposition(h, samples);
   JobParams p = *pk.base;

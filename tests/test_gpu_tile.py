@@ -73,7 +73,7 @@ def test_tile_population_edge_lattices(torch, B, empty):
     cfg = synth.config("pusht", n_steps=20, n_layer=2)
     U, T, N = 6, 20, 11
     W = synth.make_weights(cfg, 0)
-    P = 40                            # enough lattices that tiles are the faster choice
+    P = 40
     lat = np.zeros((P, U, T), np.uint8)
     lat[0, 0, 0] = 1                  # the first cell only
     lat[1, U - 1, T - 1] = 1          # the last cell only
@@ -94,13 +94,12 @@ def test_tile_population_edge_lattices(torch, B, empty):
     full = x[4]
     want = np.linalg.norm((x - full[None]).reshape(P, N, -1), axis=2).mean(1)
     assert np.allclose(dev, want, rtol=1e-4, atol=1e-5)
-    # a few short lattices are faster on clusters, whether they come from the host or the device
-    x2, _ = ev.population(torch.from_numpy(obs).cuda(), torch.from_numpy(noise).cuda(), lat[:11])
-    assert not on_tiles(ev) and ev.last_call()["path"] == "cluster"
-    x3, _ = ev.population(torch.from_numpy(obs).cuda(), torch.from_numpy(noise).cuda(), torch.from_numpy(lat[:11]).cuda())
-    assert not on_tiles(ev) and torch.equal(x2, x3)
-    for p in (0, 5, 9):
-        close(x2[p].cpu().numpy()[idx], O.denoise(W, cfg, obs[idx], noise[:, idx], lat[p], policy=empty), f"{p} on clusters")
+    # a few short lattices stay on tiles (132 samples), which keep the partial sums that cross
+    # a cluster in bf16 in fp32, with the same bits wherever the lattices live
+    for lattices in (lat[:11], torch.from_numpy(lat[:11]).cuda()):
+        x2, _ = ev.population(torch.from_numpy(obs).cuda(), torch.from_numpy(noise).cuda(), lattices)
+        assert on_tiles(ev)
+        assert np.array_equal(x2.cpu().numpy(), x[:11])
 
 
 def test_tile_lattice_forms(torch, B):
