@@ -164,7 +164,7 @@ evo_status evo_schedule_fixed_interval(int32_t n_units, int32_t T, int32_t M, ui
 /* Debug variant of evo_denoise that also records the residual added at every
  * lattice cell: trace device [T][3L][N][H][E] float32 (refreshed cells: r_{b,t};
  * skipped cells: the cached c_b as stored; empty cache under ZERO: 0).  Takes
- * the same path (one cluster per job, or batch-wide) as evo_denoise would. */
+ * the same path (one cluster per job, tile kernel, or batch-wide) as evo_denoise would. */
 evo_status evo_denoise_trace(evo_handle* h, const float* obs, const float* noise,
                              const uint8_t* S, int32_t S_rows, int32_t N,
                              float* out_actions, float* trace, void* stream);

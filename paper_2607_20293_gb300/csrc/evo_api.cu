@@ -1012,7 +1012,7 @@ bool sparse_for_tile(const evo_handle* h, long long samples, int S_rows) {
 // lattice: out holds the samples of all, the last is a population's reference
 // (actions: the candidates' copy or null, dev: their deviation).
 evo_status run_tile(evo_handle* h, const float* obs, const float* noise, float* out, int N, int n_sched, int S_rows,
-                    cudaStream_t st, float* actions = nullptr, float* dev = nullptr) {
+                    cudaStream_t st, float* actions = nullptr, float* dev = nullptr, float* trace = nullptr) {
   long long n = 0;
   EVO_CUDA(wide_condition(h->wide, obs, N, nullptr, true, h->status, true, st, &n));
   TileCall c{};
@@ -1028,6 +1028,7 @@ evo_status run_tile(evo_handle* h, const float* obs, const float* noise, float* 
   c.kv_time = wide_tile_kv_time(h->wide);
   c.stab = h->stab;
   c.out = out;
+  c.trace = trace;
   c.n_sched = n_sched;
   c.per_sched = N;
   c.obs_mod = N;
@@ -1059,7 +1060,8 @@ evo_status run(evo_handle* h, const float* obs, const float* noise, const uint8_
   if (use_wide(h, N)) {
     const evo_status s = stage_wide(h, S, 1, S_rows, false, st);
     if (s != EVO_OK) return s;
-    if (!trace && h->tile && !sparse_for_tile(h, N, S_rows)) return run_tile(h, obs, noise, out, N, 1, S_rows, st);
+    if (h->tile && !sparse_for_tile(h, N, S_rows))
+      return run_tile(h, obs, noise, out, N, 1, S_rows, st, nullptr, nullptr, trace);
     h->last_cond_kernels = 0;                  // the batch-wide sequence computes kv_obs itself
     EVO_CUDA(launch_wide(h, obs, noise, out, N, N, 1, S_rows, st, trace));
     return finish(h, st);

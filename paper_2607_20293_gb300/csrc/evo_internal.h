@@ -319,6 +319,7 @@ struct TileCall {
   const float *noise, *stab;
   const __nv_bfloat16 *kv_obs, *kv_time;   // [obs_mod][n_obs][L][2E], [T][L][2E], head dims in tile_kv_column order
   float* out;                     // [n_sched * per_sched][H][A]
+  float* trace;                   // or null: [T][U][samples][H][E] (evo_denoise_trace)
   const uint64_t* mask;           // wide_masks
   const int* order;               // or null: the order in which the lattices are taken
   int n_sched, per_sched, obs_mod;

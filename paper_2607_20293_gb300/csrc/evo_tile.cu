@@ -124,6 +124,8 @@ struct TileParams {
   const __nv_bfloat16* kv_obs;     // [obs_mod][n_obs][L][512]
   uint4* cache;                    // [grid][U][16][256]: thread-ordered bf16
   float* out;                      // [samples][16][A]
+  float* trace;                    // TRACE: [T][U][rows][256], what every cell adds to the stream
+  long long rows;                  // rows of the call
   float scale;
   int* status;
   long long wait_limit;
@@ -368,6 +370,8 @@ __device__ __forceinline__ int lattice_of(const TileParams& p, int j) {
   return p.order ? __ldg(p.order + k) : k;
 }
 
+// TRACE: the debug variant, which also stores every cell's residual
+template <bool TRACE>
 __global__ void __launch_bounds__(TTHREADS, 1) tile_kernel(const TileParams p) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -625,6 +629,17 @@ __global__ void __launch_bounds__(TTHREADS, 1) tile_kernel(const TileParams p) {
       for (int t = 0; t < p.T; ++t) {
         const uint64_t ref = __ldg(mk + 2 * t), val = __ldg(mk + 2 * t + 1);
         uint64_t rest = ref, skip = ~ref & val;
+        // the lane's place in cell (t, k): columns 2 tq, + 1 of row g
+        auto trace_cell = [&](int k) {
+          return p.trace + (((long long)t * p.U + k) * p.rows + (long long)sample * TH + g) * TE + 2 * tq;
+        };
+        if (TRACE && live)
+          for (int k = 0; k < p.U; ++k)                 // a cache never written adds nothing
+            if (!((ref | val) >> k & 1ull))
+              for (int i = 0; i < 32; ++i) {
+                *reinterpret_cast<float2*>(trace_cell(k) + 8 * i) = make_float2(0.f, 0.f);
+                *reinterpret_cast<float2*>(trace_cell(k) + 8 * TE + 8 * i) = make_float2(0.f, 0.f);
+              }
         for (;;) {
           const int b = rest ? __ffsll((long long)rest) - 1 : p.U;
           // Eq. 1: the skipped units before b whose cache holds a value
@@ -646,6 +661,13 @@ __global__ void __launch_bounds__(TTHREADS, 1) tile_kernel(const TileParams p) {
                 a[1][c] = add2(a[1][c], bf2(raw[i].y));
                 a[0][c + 1] = add2(a[0][c + 1], bf2(raw[i].z));
                 a[1][c + 1] = add2(a[1][c + 1], bf2(raw[i].w));
+                if (TRACE && live) {
+                  float* tr = trace_cell(k) + 8 * c;
+                  *reinterpret_cast<float2*>(tr) = bf2(raw[i].x);
+                  *reinterpret_cast<float2*>(tr + 8 * TE) = bf2(raw[i].y);
+                  *reinterpret_cast<float2*>(tr + 8) = bf2(raw[i].z);
+                  *reinterpret_cast<float2*>(tr + 8 * TE + 8) = bf2(raw[i].w);
+                }
               }
             }
           }
@@ -895,6 +917,11 @@ __global__ void __launch_bounds__(TTHREADS, 1) tile_kernel(const TileParams p) {
                 w[2 * e + 1] = pk2(r1.x, r1.y);
                 a[0][8 * c + i + e] = add2(a[0][8 * c + i + e], r0);
                 a[1][8 * c + i + e] = add2(a[1][8 * c + i + e], r1);
+                if (TRACE && live) {
+                  float* tr = trace_cell(b) + 8 * (8 * c + i + e);
+                  *reinterpret_cast<float2*>(tr) = r0;
+                  *reinterpret_cast<float2*>(tr + 8 * TE) = r1;
+                }
               }
               dst[(4 * c + (i >> 1)) * TCT] = make_uint4(w[0], w[1], w[2], w[3]);
             }
@@ -1122,7 +1149,8 @@ int tile_create(TileState** out, const evo_config* c, const float* weights, cons
     return fail(EVO_ERR_OOM);
   if (cudaMemcpy(s->wpack, wp.data(), wp.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(s->vec, vec.data(), vec.size() * 4, cudaMemcpyHostToDevice) != cudaSuccess ||
-      cudaFuncSetAttribute(tile_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TILE_SMEM) != cudaSuccess)
+      cudaFuncSetAttribute(tile_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, TILE_SMEM) != cudaSuccess ||
+      cudaFuncSetAttribute(tile_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, TILE_SMEM) != cudaSuccess)
     return fail(EVO_ERR_CUDA);
   *out = s;
   return EVO_OK;
@@ -1162,11 +1190,16 @@ cudaError_t tile_run(const TileState* s, const TileCall& c) {
   p.kv_obs = c.kv_obs;
   p.cache = s->cache;
   p.out = c.out;
+  p.trace = c.trace;
+  p.rows = (long long)c.n_sched * c.per_sched * TH;
   p.scale = 0.125f;               // 1 / sqrt(64)
   p.status = c.status;
   p.wait_limit = WAIT_CYCLES_DEFAULT;
   const int grid = std::min(p.n_jobs, s->cache_slots);
-  tile_kernel<<<grid, TTHREADS, TILE_SMEM, c.st>>>(p);
+  if (c.trace)
+    tile_kernel<true><<<grid, TTHREADS, TILE_SMEM, c.st>>>(p);
+  else
+    tile_kernel<false><<<grid, TTHREADS, TILE_SMEM, c.st>>>(p);
   return cudaGetLastError();
 }
 

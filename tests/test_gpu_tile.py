@@ -10,6 +10,7 @@ actions (bf16 mode), on sampled chunks."""
 import numpy as np
 import pytest
 
+from eq1_trace import check_reuse
 from oracle import evo_oracle as O
 from paper_2607_20293_gb300 import synth
 
@@ -124,6 +125,35 @@ def test_tile_lattice_forms(torch, B):
             ev.denoise(obs, noise, lattice, out=out)
         assert e.value.code == B.ERR_SCHEDULE
     assert torch.all(out == 5.0) and ev.status() == B.OK
+
+
+@pytest.mark.parametrize("empty", ["zero", "force"])
+def test_tile_trace_takes_the_tile_path(torch, B, empty):
+    # the traced call runs where the untraced one does and gives its actions bit for bit; a cell that
+    # is skipped adds the stored bf16 value (Eq. 1), one that is refreshed its own output
+    cfg = synth.config("pusht", n_steps=10, n_layer=2)
+    n, U, T = 131, 6, 10                       # a last tile of 3 samples
+    W = synth.make_weights(cfg, 0)
+    S = synth.bernoulli_schedule(U, T, 0.5, 97)
+    S[2] = 0                                   # a unit that is never refreshed
+    S[4, :3], S[4, 3] = 0, 1                   # one whose cache stays empty at first
+    obs_h, noise_h = synth.make_obs(cfg, n, 98), synth.make_noise(cfg, n, 99)
+    obs, noise = torch.from_numpy(obs_h).cuda(), torch.from_numpy(noise_h).cuda()
+    ev = B.Evo(cfg, W, n, empty=empty)
+    want = ev.denoise(obs, noise, S)
+    assert on_tiles(ev)
+    tr = torch.full((T, U, n, 16, 256), float("nan"), device="cuda")
+    got = ev.denoise(obs, noise, S, trace=tr)
+    assert on_tiles(ev) and torch.equal(got, want) and ev.status() == B.OK
+    tr = tr.cpu().numpy()
+    assert np.all(np.isfinite(tr))
+    assert check_reuse(tr, S, bf16=True, force=empty == "force") > 0
+    idx, ref = [0, 8, n - 1], {}
+    O.denoise(W, cfg, obs_h[idx], noise_h[:, idx], S, policy=empty, trace=ref)
+    # (3 % of the largest: the bound on final actions, relative)
+    top = max(np.max(np.abs(v)) for _, v in ref.values() if v is not None)
+    for (b, t), (_, v) in ref.items():
+        assert np.max(np.abs(tr[t, b][idx] - (0.0 if v is None else v))) <= TOL * top, (b, t)
 
 
 @pytest.mark.parametrize("n", [109, 127])
