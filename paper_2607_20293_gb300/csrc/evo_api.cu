@@ -995,17 +995,27 @@ bool use_wide(const evo_handle* h, long long samples) {
 // fp32.  (109 .. 127 samples of the 10-action policy at refresh fraction 0.125 /
 // 1.0 would take 7.1 / 34.5 ms on tiles and take 9.4 / 45.6 in four rounds of the
 // 36 clusters.)
-// Where the batch-wide path is the other choice, it stays ahead on one sparse
-// lattice for few samples (a tile adds the skipped units' caches 64 KiB at a
-// time on one SM): 128 / 176 / 208 samples of the 10-action policy at fraction
-// 0.05 take 3.3 / 3.6 / 3.7 ms there and 4.1 on tiles, at 0.08 5.0 / 5.5 / 5.7
-// and 5.5, at 0.125 7.1 / 7.8 / 8.1 and 7.1.
-bool sparse_for_tile(const evo_handle* h, long long samples, int S_rows) {
-  if (samples >= 224) return false;
+// On one lattice, the batch-wide path stays ahead where few cells a step are
+// refreshed for few samples: a step of a tile costs its skipped units' caches,
+// 64 KiB each on one SM, whatever the batch, a launch its latency.  The line lies
+// at the refreshed cells per step where both took the same time: at 2, 4, 8, 12
+// layers 2.7, 3.6, 4.8, 5.4 for 128 samples and 1.5, 1.7, 2.1, 2.9 for 224, and
+// about as many with 2 actions instead of 10 and 20 steps instead of 100.  8
+// layers, 10 actions, 100 steps, ms on tiles / batch-wide with buffers that change
+// / replayed:
+//   samples  1.3 cells a step      3.3                   6.3
+//   128      4.05 / 3.10 / 2.95    6.96 / 6.60 / 6.26    11.0 / 11.8 / 11.1
+//   224      4.11 / 3.60 / 3.50    7.06 / 7.69 / 7.41    11.1 / 13.7 / 13.2
+//   256      4.12 / 4.43 / 4.32    7.06 / 8.93 / 8.66    11.1 / 15.4 / 15.0
+// and with 0.26 cells a step 2.13 / 1.94 at 304 samples, 2.16 / 2.12 at 400, 2.22 /
+// 2.99 at 608.  Calls of more tiles than SMs stay ahead as well: 1,224 samples (153
+// tiles) 5.1 / 5.5 with 0.26, 16.1 / 22.6 with 3.3, 68.9 / 117 at full refresh.
+bool sparse_for_tile(const evo_handle* h, int samples, int S_rows) {
   const size_t n = (size_t)S_rows * h->T;
-  size_t cells = 0;
+  double cells = 0.0;
   for (size_t i = 0; i < n; ++i) cells += h->last_sched[i];
-  return 8 * cells < n;
+  const double per_step = cells * (h->U / S_rows) / h->T;
+  return per_step < (samples < 240 ? (2.2 + 0.1 * h->U) * (316 - samples) / 188 : samples < 500 ? 0.4 : 0.0);
 }
 
 // The tile path over n_sched staged lattices of N samples each.  More than one

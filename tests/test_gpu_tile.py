@@ -46,13 +46,13 @@ def close(got, want, what=""):
     assert err <= TOL, f"{what}: max-abs {err:.3e}"
 
 
-# 128 = 16 full tiles, 129 = a tile of one sample, 133 = a tile of 5, 143 = of 7
+# 128 = 16 full tiles, 129 = a last tile of one sample, 506 = of 2, 133 = of 5, 231 = of 7
 @pytest.mark.parametrize("n,over,frac", [
     (133, {}, 0.3),
     (128, dict(action_dim=16, n_obs=7, obs_dim=30), 1.0),
-    (129, dict(action_dim=1, n_obs=1), 0.2),
-    (143, dict(sampler="ddim", n_layer=1), 0.5),
-    (230, dict(n_layer=2, action_dim=5), 0.05),
+    (129, dict(action_dim=1, n_obs=1), 0.3),
+    (231, dict(sampler="ddim", n_layer=1), 0.5),
+    (506, dict(n_layer=2, action_dim=5), 0.05),
 ])
 def test_tile_matches_oracle(torch, B, n, over, frac):
     cfg = synth.config("pusht", n_steps=20, **over)
@@ -111,7 +111,7 @@ def test_tile_lattice_forms(torch, B):
     W = synth.make_weights(cfg, 0)
     obs = torch.from_numpy(synth.make_obs(cfg, n, 91)).cuda()
     noise = torch.from_numpy(synth.make_noise(cfg, n, 92)).cuda()
-    S = synth.bernoulli_schedule(2, 20, 0.4, 93)
+    S = synth.bernoulli_schedule(2, 20, 0.7, 93)
     ev = B.Evo(cfg, W, n)
     want = ev.denoise(obs, noise, np.repeat(S, 3, axis=0)).cpu().numpy()
     assert on_tiles(ev)
@@ -127,12 +127,38 @@ def test_tile_lattice_forms(torch, B):
     assert torch.all(out == 5.0) and ev.status() == B.OK
 
 
+# 2 layers: the line lies at 2.8 refreshed cells a step for 128 samples, at 1.15 for 239,
+# 0.4 from 240 to 499 and 0 from 500 on
+@pytest.mark.parametrize("n,cells,tiles", [(128, 27, False), (128, 29, True), (239, 11, False), (239, 12, True),
+                                           (240, 3, False), (240, 4, True), (499, 3, False), (500, 0, True)])
+def test_one_sparse_lattice_runs_batch_wide(torch, B, n, cells, tiles):
+    cfg = synth.config("pusht", n_steps=10, n_layer=2)
+    W = synth.make_weights(cfg, 0)
+    S = np.zeros((60,), np.uint8)
+    S[np.random.default_rng(n).choice(60, cells, replace=False)] = 1
+    S = S.reshape(6, 10)
+    obs, noise = synth.make_obs(cfg, n, 74), synth.make_noise(cfg, n, 75)
+    d_obs, d_noise = torch.from_numpy(obs).cuda(), torch.from_numpy(noise).cuda()
+    ev = B.Evo(cfg, W, n)
+    got = ev.denoise(d_obs, d_noise, S)
+    assert ev.last_call()["path"] == ("cluster" if tiles else "wide")
+    assert torch.equal(ev.denoise(d_obs, d_noise, torch.from_numpy(S).cuda()), got)
+    assert ev.last_call()["path"] == ("cluster" if tiles else "wide")
+    idx = [0, n - 1]
+    close(got.cpu().numpy()[idx], O.denoise(W, cfg, obs[idx], noise[:, idx], S), f"n={n} cells={cells}")
+    if cells % 3 == 0:                         # the same cells as rows of layers
+        L = np.zeros((2, 10), np.uint8)
+        L.reshape(-1)[:cells // 3] = 1
+        ev.denoise(d_obs, d_noise, L)
+        assert ev.last_call()["path"] == ("cluster" if tiles else "wide")
+
+
 @pytest.mark.parametrize("empty", ["zero", "force"])
 def test_tile_trace_takes_the_tile_path(torch, B, empty):
     # the traced call runs where the untraced one does and gives its actions bit for bit; a cell that
     # is skipped adds the stored bf16 value (Eq. 1), one that is refreshed its own output
     cfg = synth.config("pusht", n_steps=10, n_layer=2)
-    n, U, T = 131, 6, 10                       # a last tile of 3 samples
+    n, U, T = 243, 6, 10                       # a last tile of 3 samples
     W = synth.make_weights(cfg, 0)
     S = synth.bernoulli_schedule(U, T, 0.5, 97)
     S[2] = 0                                   # a unit that is never refreshed
