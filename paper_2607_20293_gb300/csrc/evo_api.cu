@@ -786,8 +786,12 @@ evo_status evo_create(const float* weights, size_t n_floats, const evo_config* c
     const int ws = wide_create(&h->wide, cfg, weights, h->wf32, h->woff, (long long)max_batch * H, max_batch + 1);
     if (ws == EVO_ERR_OOM || ws == EVO_ERR_CUDA) return fail((evo_status)ws);
     if (cfg->wide_rows > 0) h->wide_rows = cfg->wide_rows;
-    // the path is the library's choice: no decomposition or batch-wide threshold is asked for
-    if (ws == EVO_OK && cfg->wide_rows == 0 && cfg->cluster == 0 && cfg->job_samples <= 0 && tile_supported(cfg)) {
+    // with a cluster of 4 at hand the cluster path stays ahead of the batch-wide
+    // one up to about 2048 action-token rows
+    else if (h->n_alt > 0 && h->alt[h->n_alt - 1].base.C <= 4) h->wide_rows = 2048;
+    // the path is the library's choice (no decomposition or batch-wide threshold is asked for), and some call reaches it
+    if (ws == EVO_OK && cfg->wide_rows == 0 && cfg->cluster == 0 && cfg->job_samples <= 0 && tile_supported(cfg) &&
+        (long long)max_batch * H >= h->wide_rows) {
       int ts = tile_create(&h->tile, cfg, weights, h->woff, max_batch);
       if (ts == EVO_OK) ts = wide_tile_kv(h->wide, weights, h->kv_time);
       if (ts != EVO_OK) return fail((evo_status)ts);
@@ -825,9 +829,6 @@ evo_status evo_create(const float* weights, size_t n_floats, const evo_config* c
     q.cache = p.cache;
     q.status = p.status;
   }
-  // with a cluster of 4 at hand the cluster path stays ahead of the batch-wide
-  // one up to about 2048 action-token rows
-  if (cfg->wide_rows == 0 && h->n_alt > 0 && h->alt[h->n_alt - 1].base.C <= 4) h->wide_rows = 2048;
   *out = h;
   return EVO_OK;
 }

@@ -182,6 +182,27 @@ def test_tile_trace_takes_the_tile_path(torch, B, empty):
         assert np.max(np.abs(tr[t, b][idx] - (0.0 if v is None else v))) <= TOL * top, (b, t)
 
 
+def test_handles_too_small_for_tiles_hold_nothing_of_them(torch, B):
+    # a handle whose largest call stays below the threshold takes no more device
+    # memory than one whose threshold is fixed, which never has a tile path (its
+    # packed weights alone are 7.3 MB at 8 layers)
+    cfg = synth.config("pusht")
+    W = synth.make_weights(cfg, 0)
+
+    def held(n, **kw):
+        torch.cuda.synchronize()
+        before = torch.cuda.mem_get_info()[0]
+        ev = B.Evo(cfg, W, n, **kw)
+        torch.cuda.synchronize()
+        used = before - torch.cuda.mem_get_info()[0]
+        ev.close()
+        return used
+
+    held(128), held(127, wide_rows=2048)       # the kernels' modules are loaded
+    assert held(127) == held(127, wide_rows=2048)
+    assert held(128) > held(128, wide_rows=2048) + (7 << 20)
+
+
 @pytest.mark.parametrize("n", [109, 127])
 def test_calls_below_the_tile_threshold_stay_on_clusters(torch, B, n):
     # the cluster path's condition kernels and head keep their operands in fp32:
