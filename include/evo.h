@@ -234,8 +234,10 @@ evo_status evo_check_guards(evo_handle* h);
 /* Synchronizes the handle's last stream, returns and clears the device status word. */
 evo_status evo_get_status(evo_handle* h);
 
-/* Launch geometry chosen at create: CTAs per job cluster, samples per job,
- * clusters resident at once, dynamic shared memory per CTA (bytes). */
+/* Launch geometry of the last cluster or tile launch (before any: the one
+ * chosen at create): CTAs per job cluster (1: a block of the tile kernel),
+ * samples per job, clusters (blocks) that can be resident at once, dynamic
+ * shared memory per CTA (bytes). */
 evo_status evo_get_launch_info(const evo_handle* h, int32_t* cluster, int32_t* job_samples,
                                int32_t* max_clusters, int32_t* smem_bytes);
 

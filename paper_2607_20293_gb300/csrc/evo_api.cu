@@ -1056,7 +1056,7 @@ evo_status run_tile(evo_handle* h, const float* obs, const float* noise, float* 
   if (actions)
     EVO_CUDA(cudaMemcpyAsync(actions, out, (size_t)P * N * HA * 4, cudaMemcpyDeviceToDevice, st));
   h->last_base = &h->tile_base;
-  h->last_mc = n_sched * ((N + 7) / 8);
+  h->last_mc = h->num_sms;                     // a block per SM at a time
   h->last_path = 0;
   h->last_kernels = n;
   return finish(h, st);

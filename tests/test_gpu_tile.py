@@ -63,6 +63,8 @@ def test_tile_matches_oracle(torch, B, n, over, frac):
     ev = B.Evo(cfg, W, n)
     got = ev.denoise(torch.from_numpy(obs).cuda(), torch.from_numpy(noise).cuda(), S).cpu().numpy()
     assert on_tiles(ev)
+    # the blocks that are resident at once, one per SM, however many tiles the call has
+    assert ev.launch_info()["max_clusters"] == torch.cuda.get_device_properties(0).multi_processor_count
     idx = [0, 7, 8, n - 2, n - 1]
     close(got[idx], O.denoise(W, cfg, obs[idx], noise[:, idx], S), f"n={n}")
     assert ev.status() == B.OK
