@@ -1209,11 +1209,13 @@ cudaError_t wide_launch(WideState* w, const WideCall& c, cudaStream_t st) {
   // Programmatic dependent launch hides the gap between kernels: 10 steps at full
   // refresh, n_emb 512, 50 samples 10.6 -> 8.7 ms, 1,024 48.3 -> 45.5 (100 steps
   // at 0.125 88.1 -> 86.7).  In a replayed graph the gaps of the largest batches
-  // are hidden without it: 1,024 at 0.125 83.8 ms, and 86.1 with it.
-  const bool captured = w->cap_stream && st == w->cap_stream;
-  const bool pdl = !captured || R < GRAPH_PDL_MAX_ROWS;
+  // are hidden without it, in the handle's own capture and in a caller's: 1,024 at
+  // 0.125 83.8 ms, and 86.1 with it.
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  cudaError_t e = cudaStreamIsCapturing(st, &cap);
+  if (e != cudaSuccess) return e;
+  const bool pdl = cap == cudaStreamCaptureStatusNone || R < GRAPH_PDL_MAX_ROWS;
   long long n = 0;
-  cudaError_t e;
 #define WCK(x)                    \
   do {                            \
     e = (x);                      \

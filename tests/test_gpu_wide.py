@@ -213,3 +213,36 @@ def test_wide_small_tiles_of_the_output_projections(torch, B, n):
     # off by more (x0 = (x - s eps) / sqrt(abar), a factor 7 at the first step, then
     # few steps to correct it: 0.031 at n = 77 on the 128-column tiles)
     assert np.linalg.norm(got[idx] - want) <= 1e-2 * np.linalg.norm(want)
+
+
+# 32,736 rows and 32,768: a captured sequence, the caller's like the handle's own, has
+# programmatic launches only below the latter
+@pytest.mark.parametrize("n,programmatic", [(1023, True), (1024, False)])
+def test_callers_capture_follows_the_replay_rule(torch, B, n, programmatic):
+    import ctypes
+    cfg = synth.config("scale1024", n_steps=2, n_layer=1)
+    ev = B.Evo(cfg, synth.make_weights(cfg, 0), n)
+    obs = torch.from_numpy(synth.make_obs(cfg, n, 64)).cuda()
+    noise = torch.from_numpy(synth.make_noise(cfg, n, 65)).cuda()
+    S = np.ones((3, 2), np.uint8)
+    want = ev.denoise(obs, noise, S)
+    assert ev.last_call()["path"] == "wide"
+    out = torch.zeros_like(want)
+    torch.cuda.synchronize()
+    rt = ctypes.CDLL("libcudart.so.13")
+    st, graph, exec_ = torch.cuda.Stream(), ctypes.c_void_p(), ctypes.c_void_p()
+    handle = ctypes.c_void_p(st.cuda_stream)
+    assert rt.cudaStreamBeginCapture(handle, 2) == 0           # relaxed
+    ev.denoise(obs, noise, S, out=out, stream=st)              # (the lattice is staged already)
+    assert rt.cudaStreamEndCapture(handle, ctypes.byref(graph)) == 0
+    k = ctypes.c_size_t(4096)
+    src, dst = (ctypes.c_void_p * k.value)(), (ctypes.c_void_p * k.value)()
+    data = (ctypes.c_uint8 * (8 * k.value))()                  # cudaGraphEdgeData: from_port, to_port, type, reserved
+    assert rt.cudaGraphGetEdges(graph, src, dst, data, ctypes.byref(k)) == 0
+    kinds = [data[8 * i + 2] for i in range(k.value)]
+    assert len(kinds) > 10 and (sum(kinds) > 10) == programmatic, kinds
+    assert rt.cudaGraphInstantiate(ctypes.byref(exec_), graph, ctypes.c_ulonglong(0)) == 0
+    assert rt.cudaGraphLaunch(exec_, handle) == 0
+    torch.cuda.synchronize()
+    assert torch.equal(out, want) and ev.status() == B.OK
+    assert rt.cudaGraphExecDestroy(exec_) == 0 and rt.cudaGraphDestroy(graph) == 0
