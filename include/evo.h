@@ -262,7 +262,8 @@ evo_status evo_get_last_call(const evo_handle* h, int32_t* path, int64_t* kernel
  *                      distributions (mean |sorted a_t - sorted a_t'|); n a power of two <= 16384
  *   d       device [U][T] fp32 (output)
  *   scratch device, evo_redundancy_scratch_bytes(...) bytes, caller-owned
- * 2 <= T <= 128.  Asynchronous on the stream; deterministic. */
+ * 2 <= T <= 128.  Asynchronous on the stream; deterministic: every sum runs in
+ * index order, so a unit's map does not depend on what else shares the call. */
 enum { EVO_METRIC_COSINE = 0, EVO_METRIC_MSE = 1, EVO_METRIC_L1 = 2, EVO_METRIC_W1 = 3 };
 size_t evo_redundancy_scratch_bytes(int32_t T, int32_t U, int32_t N, int32_t n, int32_t metric);
 evo_status evo_redundancy_map(const float* trace, int32_t T, int32_t U, int32_t N, int32_t n, int32_t metric,

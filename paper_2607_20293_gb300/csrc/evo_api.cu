@@ -984,18 +984,22 @@ bool use_wide(const evo_handle* h, long long samples) {
   return h->wide && samples * h->H >= h->wide_rows && samples * h->H <= wide_rows_capacity(h->wide);
 }
 
-// The tile path serves calls that the batch-wide path would serve too, every
-// population among them: a lattice's refreshed cells are work for its own tiles
-// there, and launches over all rows here.  Push-T shaped, tiles / batch-wide: 12
-// candidates x 11 observations of 5 .. 60 % density 33.7 / 49.5 ms, 127 x 1 33.9 /
-// 58.8, 16 x 16 33.7 / 53.4, 64 x 16 33.8 / 97.5.  (4-CTA clusters would take
-// 18.9 / 17.4 / 37.2 / 133, but pass the residual stream's LayerNorm input and the
-// second GEMM's partial sums on in bf16, which both of these keep in fp32.)  Both
-// round the same values (the condition path's operands, the head's weights) to
-// bf16, where the cluster path, which takes all smaller calls, keeps them in
-// fp32.  (109 .. 127 samples of the 10-action policy at refresh fraction 0.125 /
-// 1.0 would take 7.1 / 34.5 ms on tiles and take 9.4 / 45.6 in four rounds of the
-// 36 clusters.)
+// The tile path serves calls that the batch-wide path would serve too, and only
+// those: both round the same values (the condition path's operands, the head's
+// weights) to bf16, where the cluster path, which takes all smaller calls, keeps
+// them in fp32.  (109 .. 127 samples of the 10-action policy at refresh fraction
+// 0.125 / 1.0 would take 7.1 / 34.5 ms on tiles and take 9.4 / 45.6 in four rounds
+// of the 36 clusters.)
+//
+// Every population is among them: a lattice's refreshed cells are work for its
+// own tiles on the one path and launches over all rows on the other.  Push-T
+// shaped, tiles / batch-wide: 12 candidates x 11 observations of 5 .. 60 % density
+// 33.7 / 49.5 ms, 127 x 1 33.9 / 58.8, 16 x 16 33.7 / 53.4, 64 x 16 33.8 / 97.5,
+// 2,000 x 1 204 / 211.  (4-CTA clusters would take 18.9 / 17.4 / 37.2 / 133 / 240,
+// but pass the LayerNorm input and the second GEMM's partial sums on in bf16, which
+// the other two keep in fp32: against 64 bits the actions of 12 x 11 are off by
+// 0.0021 there and 0.0013 here.)
+//
 // On one lattice, the batch-wide path stays ahead where few cells a step are
 // refreshed for few samples: a step of a tile costs its skipped units' caches,
 // 64 KiB each on one SM, whatever the batch, a launch its latency.  The line lies

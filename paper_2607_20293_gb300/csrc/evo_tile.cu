@@ -49,7 +49,7 @@
 // SM sub-partition (the register file holds no more of them beside the stream:
 // with sixteen warps of half a row the compiler spills it).  A unit takes about
 // 14 us.  64 candidates x 16 observations and their reference (n_emb 256, 8
-// layers, 100 steps): 97.5 ms batch-wide -> 34.6 ms, the reference's 2,400
+// layers, 100 steps): 97.5 ms batch-wide -> 33.9 ms, the reference's 2,400
 // units; 300 samples at refresh fraction 0.125: 10.3 -> 7.1 ms.
 //
 // Warps 0-7 compute, warp 8 streams weights, warp 9 issues the MMAs (10 and 11
