@@ -492,7 +492,7 @@ def run_redundancy(args, rank):
                    "l2": "flushed between timed calls (256 MiB write)"},
         "map_ms": maps, "trace_collection_ms": trace_ms,
         "guided": {"schedules": P, "K": K, "ms": guided_ms, "schedules_per_s": P / (guided_ms * 1e-3)},
-        "roofline": {"bound": "alu", "kernel": "pair_kernel (cosine)", "achieved": achieved, "peak": peak,
+        "roofline": {"bound": "alu", "kernel": "evo::ordered_pair_kernel (cosine)", "achieved": achieved, "peak": peak,
                      "unit": "TFLOP/s", "frac": achieved / peak, "traffic": None,
                      "peak_source": f"{sm} SMs x {FP32_LANES_PER_SM} FP32 lanes x 2 FLOP x {mhz:.0f} MHz"},
         "clocks": clk,

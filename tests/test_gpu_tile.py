@@ -187,7 +187,7 @@ def test_tile_trace_takes_the_tile_path(torch, B, empty):
 def test_handles_too_small_for_tiles_hold_nothing_of_them(torch, B):
     # a handle whose largest call stays below the threshold takes no more device
     # memory than one whose threshold is fixed, which never has a tile path (its
-    # packed weights alone are 7.3 MB at 8 layers)
+    # packed weights alone are 14.7 MB at 8 layers)
     cfg = synth.config("pusht")
     W = synth.make_weights(cfg, 0)
 
@@ -202,7 +202,7 @@ def test_handles_too_small_for_tiles_hold_nothing_of_them(torch, B):
 
     held(128), held(127, wide_rows=2048)       # the kernels' modules are loaded
     assert held(127) == held(127, wide_rows=2048)
-    assert held(128) > held(128, wide_rows=2048) + (7 << 20)
+    assert held(128) > held(128, wide_rows=2048) + 14_000_000
 
 
 @pytest.mark.parametrize("n", [109, 127])
